@@ -2,7 +2,8 @@
 
 A case is a dict of plain values; its "kind" names one way the library is used:
 
-  plain    gray plain Monte Carlo step: reset, transport, temperatures, escape spectrum
+  plain    gray plain Monte Carlo step: reset, transport, temperatures, escape spectrum; "repeat": the
+           bitwise repeatable form of the run (no tail kernel)
   thick    the same with the modified random walk on a very thick gray disk (optionally with the PDA)
   nongray  the same with wavelength-dependent, anisotropically scattering dust
   scatter  a step that keeps the mean-intensity tally, then the ray-traced SED with scattered light
@@ -14,10 +15,10 @@ A case is a dict of plain values; its "kind" names one way the library is used:
   rays     ray-traced SED and N-band visibilities of a disk with known temperatures
   hydro    one vertical-structure update from known temperatures
 
-What a transport step returns: the escape spectrum, and the temperatures where two runs on the same
-inputs agree on them. In very thick or non-gray disks the nearly empty cells hold the deposits of single
-packets whose paths depend on the order in which the GPU interleaves packets, so the temperature array of
-such a run says nothing about another run of the same code.
+What a transport step returns: the escape spectrum, and, of a repeatable run, the temperatures and the
+integer tallies. By default the nearly empty cells hold the deposits of single packets whose paths depend
+on when the tail kernel takes them over (and, with non-gray dust, on the order in which the GPU
+interleaves packets), so the temperature array of such a run says little about another run of the same code.
 """
 import math
 import struct
@@ -37,7 +38,7 @@ SIGMA = disks.SIGMA_SB
 def listed():
     return [
         # a small optically thin-to-moderate disk, the ordinary first run of a user (40 x 40 gray, tau 100)
-        dict(name="plain_40x40_1e6", kind="plain", nr=40, nt=40, tau=100.0, n=1_000_000),
+        dict(name="plain_40x40_1e6", kind="plain", nr=40, nt=40, tau=100.0, n=1_000_000, repeat=False),
         # a quick look at the thick disk: few packets, the call waits for its longest ones
         dict(name="thick_200x120_1e6", kind="thick", nr=200, nt=120, tau=1e6, n=1_000_000, gamma=2.0, pda=False),
         # the production run of the thick disk with MRW and PDA (the benchmark step)
@@ -47,7 +48,7 @@ def listed():
         # scattered-light SED: path-length tally kept in the run, then ray tracing with it
         dict(name="scatter_60x40_1e6", kind="scatter", nr=60, nt=40, tau=1e4, n=1_000_000, nphi=32),
         # broad-band polarization against inclination of a disk of small particles
-        dict(name="polar_60x40_1e6", kind="polar", nr=60, nt=40, tau=1e4, n=1_000_000),
+        dict(name="polar_60x40_1e6", kind="polar", nr=60, nt=40, tau=1e3, n=1_000_000),
         # a parameter sweep of uneven non-gray disks replayed from one graph
         dict(name="batch_6", kind="batch", models=6, lo=30, hi=80, tau=1e3, n=1_200_000),
         # post-processing of a saved run: non-gray temperatures and the diffusion solve on the 400 x 200 disk
@@ -77,7 +78,8 @@ def draw(rng):
                        "hydro"])
     c = dict(kind=kind)
     if kind == "plain":
-        c.update(nr=_ilog(rng, 12, 150), nt=2 * _ilog(rng, 6, 60), tau=_log(rng, 10, 1e3), n=_ilog(rng, 1e5, 2e7))
+        c.update(nr=_ilog(rng, 12, 150), nt=2 * _ilog(rng, 6, 60), tau=_log(rng, 10, 1e3), n=_ilog(rng, 1e5, 2e7),
+                 repeat=rng.random() < 0.5)
     elif kind == "thick":
         c.update(nr=_ilog(rng, 60, 300), nt=2 * _ilog(rng, 20, 90), tau=_log(rng, 1e4, 1e6), n=_ilog(rng, 5e5, 5e7),
                  gamma=rng.choice([2.0, 4.0, 10.0]), pda=False)
@@ -88,7 +90,7 @@ def draw(rng):
         c.update(nr=_ilog(rng, 20, 100), nt=2 * _ilog(rng, 10, 30), tau=_log(rng, 30, 1e4), n=_ilog(rng, 2e5, 2e6),
                  nphi=rng.randint(16, 64))
     elif kind == "polar":
-        c.update(nr=_ilog(rng, 20, 100), nt=2 * _ilog(rng, 10, 30), tau=_log(rng, 30, 1e4), n=_ilog(rng, 5e5, 3e6))
+        c.update(nr=_ilog(rng, 20, 100), nt=2 * _ilog(rng, 10, 30), tau=_log(rng, 30, 1e3), n=_ilog(rng, 2e5, 2e6))
     elif kind == "batch":
         c.update(models=rng.randint(2, 8), lo=20, hi=rng.randint(40, 120), tau=_log(rng, 1e2, 1e3),
                  n=_ilog(rng, 6e5, 2e6))
@@ -272,8 +274,9 @@ def run(s):
     kind = c["kind"]
     if kind == "plain":
         s.disk.reset()
-        s.disk.run_photons(c["n"], seed=s.seed)
-        return {"T": s.disk.temperatures()[0], "sed": s.disk.sed()}
+        s.disk.run_photons(c["n"], seed=s.seed, tail_warps=-1 if c["repeat"] else 0)
+        T, sed = s.disk.temperatures()[0], s.disk.sed()
+        return {"T": T, "tallies": list(s.disk.tallies()), "sed": sed} if c["repeat"] else {"sed": sed}
     if kind == "thick":
         s.disk.reset()
         s.disk.run_photons(c["n"], seed=s.seed, mrw=True, gamma=c["gamma"], max_events=10 ** 6)
@@ -290,7 +293,8 @@ def run(s):
         s.disk.reset()
         s.disk.run_photons(c["n"], seed=s.seed, mrw=True, gamma=2.0, max_events=10 ** 6)
         o = s.disk.raytrace(scattering=True)
-        return {"T": s.disk.temperatures()[0], "F": o["F"].astype(np.float32), "sed": s.disk.sed()}
+        s.disk.temperatures()
+        return {"F": o["F"].astype(np.float32), "sed": s.disk.sed()}
     if kind == "polar":
         s.disk.reset()
         s.disk.run_photons(c["n"], seed=s.seed, mrw=True, gamma=2.0, max_events=10 ** 6)
