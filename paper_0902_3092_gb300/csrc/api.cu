@@ -644,6 +644,21 @@ static uint64_t in_flight_cap(bool gray, double n_total, uint64_t requested) {
   return std::max<uint64_t>(32, (uint64_t)(n_total / MCRT_NONGRAY_IN_FLIGHT));
 }
 
+// Non-gray FP32 runs carry one packet per warp (transport_warp_kernel): few packets are in flight (see
+// MCRT_NONGRAY_IN_FLIGHT), so a packet that shares its warp with others only waits for them, and a warp's
+// lanes can take a flight's cells and a re-emission's table searches together. (tail_warps_per_sm = -1, the
+// form of the run whose packets all stay in the transport kernel, and polarized runs keep a packet per lane.)
+static bool one_packet_per_warp(bool gray, bool pol, const mcrt_run_opts* o) {
+  return !gray && !pol && o->tail_warps_per_sm >= 0;
+}
+
+// warps of such a launch: one packet each, at most the resident ones and max_in_flight
+static int warp_grid(uint64_t n_packets, int sms, int warps_per_sm, uint64_t max_in_flight) {
+  uint64_t g = std::min<uint64_t>(n_packets, (uint64_t)sms * std::max(1, warps_per_sm));
+  if (max_in_flight) g = std::min(g, max_in_flight);
+  return (int)std::max<uint64_t>(1, g);
+}
+
 // Queue of a batch with non-gray dust: chunks of 32 slots of one model, ordered so that every model moves
 // through its packets at the same pace (chunk k of model m at (k + 1/2) / chunks_m, ties by model), so that
 // each model has the launch's share of its packets in flight (see MCRT_NONGRAY_IN_FLIGHT in mcrt.h).
@@ -756,20 +771,27 @@ static mcrt_status run_impl(mcrt_disk* d, uint64_t n_packets, uint64_t seed, uin
       P.queue = d->queue.as<unsigned long long>();
       P.trip = d->cnt.as<unsigned long long>() + C_NCNT;
       P.want_lam = (!d->gray || o->want_sed) ? 1 : 0;
-      const int bps = pol  ? transport_blocks_per_sm_pol<float>(d->gray, block)
-                      : jt ? transport_blocks_per_sm_j<float>(d->gray, block)
-                           : transport_blocks_per_sm<float>(false, false, d->gray, block);
-      const int grid = transport_grid(n_packets, block, dev_sms, bps, in_flight_cap(d->gray, d->n_total, o->max_in_flight));
-      const bool tail = setup_pool(d, P, (unsigned)grid * block, o->tail_warps_per_sm);
-      e = pol  ? launch_transport_pol<float>(P, d->gray, grid, block, d->stream)
-          : jt ? launch_transport_j<float>(P, d->gray, grid, block, d->stream)
-               : launch_transport<float>(P, false, false, d->gray, grid, block, d->stream);
-      d->launches++;
-      if (e == cudaSuccess && tail) {
-        e = pol  ? launch_transport_tail_pol<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)
-            : jt ? launch_transport_tail_j<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)
-                 : launch_transport_tail<float>(P, false, false, d->gray, dev_sms, o->tail_warps_per_sm, d->stream);
+      const uint64_t cap = in_flight_cap(d->gray, d->n_total, o->max_in_flight);
+      if (one_packet_per_warp(d->gray, pol, o)) {
+        const int warps = warp_grid(n_packets, dev_sms, jt ? transport_warps_per_sm_j() : transport_warps_per_sm(false), cap);
+        e = jt ? launch_transport_warp_j(P, warps, d->stream) : launch_transport_warp(P, false, warps, d->stream);
         d->launches++;
+      } else {
+        const int bps = pol  ? transport_blocks_per_sm_pol<float>(d->gray, block)
+                        : jt ? transport_blocks_per_sm_j<float>(d->gray, block)
+                             : transport_blocks_per_sm<float>(false, false, d->gray, block);
+        const int grid = transport_grid(n_packets, block, dev_sms, bps, cap);
+        const bool tail = setup_pool(d, P, (unsigned)grid * block, o->tail_warps_per_sm);
+        e = pol  ? launch_transport_pol<float>(P, d->gray, grid, block, d->stream)
+            : jt ? launch_transport_j<float>(P, d->gray, grid, block, d->stream)
+                 : launch_transport<float>(P, false, false, d->gray, grid, block, d->stream);
+        d->launches++;
+        if (e == cudaSuccess && tail) {
+          e = pol  ? launch_transport_tail_pol<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)
+              : jt ? launch_transport_tail_j<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)
+                   : launch_transport_tail<float>(P, false, false, d->gray, dev_sms, o->tail_warps_per_sm, d->stream);
+          d->launches++;
+        }
       }
     }
     if (e != cudaSuccess) {
@@ -891,14 +913,18 @@ mcrt_status mcrt_run_batch(mcrt_disk* const* disks, int n, const uint64_t* n_pac
   int dev_sms = 0;
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, d->device), "attribute");
   const int block = o->block_size ? o->block_size : 128;
-  const int bps = transport_blocks_per_sm<float>(false, true, false, block);
-  const int grid = transport_grid(P.total, block, dev_sms, bps, in_flight_cap(!any_nongray, (double)q, o->max_in_flight));
+  const uint64_t cap = in_flight_cap(!any_nongray, (double)q, o->max_in_flight);
+  const bool warp = one_packet_per_warp(!any_nongray, false, o);
+  const int grid = warp ? warp_grid(P.total, dev_sms, transport_warps_per_sm(true), cap)
+                        : transport_grid(P.total, block, dev_sms,
+                                         transport_blocks_per_sm<float>(false, true, false, block), cap);
   cudaEvent_t ev0, ev1;
   CK(cudaEventCreate(&ev0), "event");
   CK(cudaEventCreate(&ev1), "event");
   CK(cudaEventRecord(ev0, d->stream), "event");
   if (q > 0) {
-    e = launch_transport<float>(P, false, true, false, grid, block, d->stream);
+    e = warp ? launch_transport_warp(P, true, grid, d->stream)
+             : launch_transport<float>(P, false, true, false, grid, block, d->stream);
     d->launches++;
     if (e != cudaSuccess) return cuda_fail(d, e, "transport launch");
   }
@@ -1210,6 +1236,7 @@ struct mcrt_batch {
   std::vector<cudaGraphNode_t> knodes;  // kernel nodes (their KParams carry the seed)
   DBuf pool, pool_ctr;                   // packets in flight at the drain, for the tail kernel
   int tail_warps = 0, sms = 0;
+  bool warp = false;                     // one packet per warp (non-gray batches)
   std::string err;
   ~mcrt_batch() {
     if (exec) cudaGraphExecDestroy(exec);
@@ -1227,6 +1254,7 @@ cudaError_t batch_launch(mcrt_batch* b, const KParams<float>& P, int block, int 
   }
   e = cudaMemsetAsync(b->queue.p, 0, 8, b->stream);
   if (e != cudaSuccess) return e;
+  if (b->warp) return launch_transport_warp(P, true, grid, b->stream);
   if (P.pool) {
     e = cudaMemsetAsync(P.pool_ctr, 0, 16, b->stream);
     if (e != cudaSuccess) return e;
@@ -1315,8 +1343,9 @@ mcrt_status mcrt_batch_create(mcrt_disk* const* disks, int n, const uint64_t* n_
   auto grid_for = [&](int block) {
     return transport_grid(b->P.total, block, sms, transport_blocks_per_sm<float>(false, true, false, block), cap);
   };
-  if (o->block_size) {
-    b->block = o->block_size;
+  b->warp = one_packet_per_warp(!any_nongray, false, o);
+  if (b->warp || o->block_size) {  // (one packet per warp: 32-thread blocks, nothing to tune)
+    b->block = b->warp ? 32 : o->block_size;
     b->refill = o->refill_interval > 0 ? o->refill_interval : 1;
   } else {
     // autotune on a short run of about 5 % of the packets (at least one per model)
@@ -1369,6 +1398,8 @@ mcrt_status mcrt_batch_create(mcrt_disk* const* disks, int n, const uint64_t* n_
     b->tune_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t_start).count();
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+  }
+  if (!o->block_size)  // a batch whose shape the library chooses starts from zero tallies
     for (int i = 0; i < n; ++i) {
       s = zero_tallies(disks[i]);
       if (s != MCRT_OK) {
@@ -1376,13 +1407,12 @@ mcrt_status mcrt_batch_create(mcrt_disk* const* disks, int n, const uint64_t* n_
         return s;
       }
     }
-  }
   b->P.refill = b->refill;
-  b->grid = grid_for(b->block);
+  b->grid = b->warp ? warp_grid(b->P.total, sms, transport_warps_per_sm(true), cap) : grid_for(b->block);
   // the tail kernel's pool: one slot per thread of the chosen launch (the autotuner ran without it)
   b->sms = sms;
   b->tail_warps = o->tail_warps_per_sm;
-  if (o->tail_warps_per_sm >= 0) {
+  if (o->tail_warps_per_sm >= 0 && !b->warp) {
     const size_t cap = (size_t)b->grid * b->block;
     if (b->pool.alloc(cap * sizeof(Pkt<float>)) == cudaSuccess && b->pool_ctr.alloc(16) == cudaSuccess) {
       b->P.pool = b->pool.as<Pkt<float>>();

@@ -48,6 +48,12 @@ int transport_blocks_per_sm(bool trace, bool batch, bool gray, int block);
 template <class R>
 cudaError_t launch_transport_tail(const KParams<R>& P, bool trace, bool batch, bool gray, int sms, int warps_per_sm,
                                   cudaStream_t st);
+// one packet per warp (FP32, non-gray runs and batches), `warps` warps in all: at most
+// transport_warps_per_sm per SM are resident
+cudaError_t launch_transport_warp(const KParams<float>& P, bool batch, int warps, cudaStream_t st);
+cudaError_t launch_transport_warp_j(const KParams<float>& P, int warps, cudaStream_t st);
+int transport_warps_per_sm(bool batch);
+int transport_warps_per_sm_j();
 // polarized transport (single disk, no event trace)
 template <class R>
 cudaError_t launch_transport_pol(const KParams<R>& P, bool gray, int grid, int block, cudaStream_t st);

@@ -25,6 +25,7 @@
 // uses the same layout, so gray trajectories of the FP64 build match it event by event.
 #pragma once
 #include "common.cuh"
+#include "flight.cuh"
 
 namespace mcrt {
 
@@ -459,22 +460,28 @@ __host__ __device__ __forceinline__ void qpos(const DevModel<R>& M, unsigned lon
 //   adjacent intervals:       D = (1 - w_old)(C[k_old+1] - C[k_old]) + w_new (C[k_new+1] - C[k_new])
 //   further apart:            D = C(T_new) - C(T_old), both interpolated
 // Below the first grid temperature (k = 0) the spectrum is the one of the first interval.
-static __host__ __device__ __noinline__ int sample_bw_rows(const float* __restrict__ C, int nl, int nT, int ko, float wo,
-                                                           int kn, float wn, float u) {
-  int mode = kn <= ko ? 0 : (kn == ko + 1 ? 1 : 2);
-  // mode 0: interval j2 weighs a2 against interval kn (j2 = kn and a2 = 0 at the grid's ends, where the
-  // first interval, from 0 K, is no derivative)
-  const float w = kn == ko ? 0.5f * (wo + wn) : wn;
-  int j2 = kn;
-  float a2 = 0.f;
-  if (w >= 0.5f && kn + 2 <= nT - 1) {
-    j2 = kn + 1;
-    a2 = w - 0.5f;
-  } else if (w < 0.5f && kn >= 2) {
-    j2 = kn - 1;
-    a2 = 0.5f - w;
+struct BwSpectrum {
+  const float* C;
+  int nl, ko, kn, j2, mode;
+  float wo, wn, a2;
+  __host__ __device__ BwSpectrum(const float* C_, int nl_, int nT, int ko_, float wo_, int kn_, float wn_)
+      : C(C_), nl(nl_), ko(ko_), kn(kn_), wo(wo_), wn(wn_) {
+    mode = kn <= ko ? 0 : (kn == ko + 1 ? 1 : 2);
+    // mode 0: interval j2 weighs a2 against interval kn (j2 = kn and a2 = 0 at the grid's ends, where the
+    // first interval, from 0 K, is no derivative)
+    const float w = kn == ko ? 0.5f * (wo + wn) : wn;
+    j2 = kn;
+    a2 = 0.f;
+    if (w >= 0.5f && kn + 2 <= nT - 1) {
+      j2 = kn + 1;
+      a2 = w - 0.5f;
+    } else if (w < 0.5f && kn >= 2) {
+      j2 = kn - 1;
+      a2 = 0.5f - w;
+    }
+    if (!((*this)(nl - 1) > 0.f)) mode = 0;
   }
-  auto D = [&](int b) -> float {
+  __host__ __device__ float operator()(int b) const {
     if (mode == 0) {
       const float* r = C + (size_t)kn * nl;
       const float* r2 = C + (size_t)j2 * nl;
@@ -488,13 +495,14 @@ static __host__ __device__ __noinline__ int sample_bw_rows(const float* __restri
     const float* ro = C + (size_t)ko * nl;
     const float* rn = C + (size_t)kn * nl;
     return ((1.f - wn) * ldg(rn + b) + wn * ldg(rn + nl + b)) - ((1.f - wo) * ldg(ro + b) + wo * ldg(ro + nl + b));
-  };
-  float tot = D(nl - 1);
-  if (!(tot > 0.f)) {
-    mode = 0;
-    tot = D(nl - 1);
   }
-  const float target = u * tot;
+  __host__ __device__ float total() const { return (*this)(nl - 1); }
+};
+
+static __host__ __device__ __noinline__ int sample_bw_rows(const float* __restrict__ C, int nl, int nT, int ko, float wo,
+                                                           int kn, float wn, float u) {
+  const BwSpectrum D(C, nl, nT, ko, wo, kn, wn);
+  const float target = u * D.total();
   int lo = -1, hi = nl - 1;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -1447,6 +1455,351 @@ __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRn
   return true;
 }
 
+// ------------------------------------------------------------------------------------------------
+// One FP32 packet per warp, its events made by the 32 lanes together (dust whose re-emission needs the
+// wavelength at once: non-gray dust, and runs that keep the mean-intensity tally). The packet's random
+// blocks are the ones it has in a lane of its own; positions along a flight come from the flight's start.
+// ------------------------------------------------------------------------------------------------
+
+// Largest index i in [lo, hi) with ok(i), given ok(lo) and ok true up to it and false after: 32 indices per
+// step (a 1024-entry table takes two dependent loads instead of ten).
+template <class F>
+__device__ __forceinline__ int warp_last(int lo, int hi, F&& ok) {
+  const int lane = (int)(threadIdx.x & 31u);
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) >> 5;
+    const int i = lo + lane * step;
+    const int n = __popc(__ballot_sync(0xffffffffu, lane == 0 || (i < hi && ok(i))));
+    lo += (n - 1) * step;
+    hi = lo + step < hi ? lo + step : hi;
+  }
+  return lo;
+}
+
+// qpos by the 32 lanes, from interval k0 on if the energy lies in it
+__device__ __forceinline__ void qpos_warp(const DevModel<float>& M, unsigned long long tally, int c, int k0, int& k,
+                                          float& w) {
+  k = 0;
+  w = 0.f;
+  if (tally == 0ull) return;
+  const float lq = fast_logf((float)tally) + ldg(M.lqm + c) + M.lq_run;
+  if (!(lq >= ldg(M.lQk + 1))) return;
+  const int nT = M.nT;
+  if (lq >= ldg(M.lQk + nT - 1)) {
+    k = nT - 2;
+    w = 1.f;
+    return;
+  }
+  if (k0 >= 1 && k0 + 1 < nT && ldg(M.lQk + k0) <= lq && lq < ldg(M.lQk + k0 + 1)) k = k0;
+  else k = warp_last(1, nT - 1, [&](int i) { return ldg(M.lQk + i) <= lq; });
+  const float a = ldg(M.lQk + k), b = ldg(M.lQk + k + 1);
+  w = (lq - a) / (b - a);
+}
+
+// smallest bin b with D(b) >= target (D(nl - 1) is taken to reach it)
+template <class F>
+__device__ __forceinline__ int warp_bin(int nl, float target, F&& D) {
+  return warp_last(-1, nl - 1, [&](int i) { return D(i) < target; }) + 1;
+}
+
+// sample_bw_rows and sample_exit_rows by the 32 lanes
+__device__ __forceinline__ int sample_bw_warp(const DevModel<float>& M, int ko, float wo, int kn, float wn, float u) {
+  const BwSpectrum S(M.cbw, M.nlam, M.nT, ko, wo, kn, wn);
+  return warp_bin(M.nlam, u * S.total(), [&](int b) { return S(b); });
+}
+__device__ __forceinline__ int sample_exit_warp(const DevModel<float>& M, int k, float w, float u) {
+  const float* X = M.cexit + (size_t)k * M.nlam;
+  auto cum = [&](int b) { return (1.f - w) * ldg(X + b) + w * ldg(X + M.nlam + b); };
+  return warp_bin(M.nlam, u * cum(M.nlam - 1), cum);
+}
+
+// The packet's flight to its next interaction point (2) or out of the grid or into a step guard (0): the
+// next 31 cells of the ray at a time (flight.cuh).
+template <bool G, bool JT>
+__device__ __forceinline__ int fly_warp(const KParams<float>& P, const DevModel<float>& M, Pkt<float>& s, Acc& acc) {
+  const int lane = (int)(threadIdx.x & 31u);
+  const unsigned full = 0xffffffffu;
+  const float chi = (G || M.gray) ? M.chi0 : M.chi[s.lam];
+  for (;;) {
+    if (++s.steps > P.max_steps) {
+      acc.err |= kErrStepGuard;
+      acc.capped++;
+      note_trip<float, WarpRng>(P, M, s, 1u);
+      return 0;
+    }
+    if (s.ir >= 0) {
+      // an interaction before the nearest face needs no crossings (d_min is at most half the shell's width)
+      const float s_int = s.alpha > 0.f ? s.tau * s.ialpha : inf_<float>();
+      bool hit = s_int < s.dsafe;
+      if (!hit && !s.xcross && 2.f * s_int < M.rf[s.ir + 1] - M.rf[s.ir]) {
+        const float dm = dmin_cell(M, s.ir, s.it, s.px, s.py, s.pz) * dsafe_margin<float>();
+        hit = s_int < dm;
+        if (hit) s.dsafe = dm;
+      }
+      if (hit) {
+        if (JT) j_flight<float, WarpRng>(M, s.ir * M.nt + s.it, s.lam, s_int);
+        s.xcross = 0;
+        s.px += s_int * s.ux;
+        s.py += s_int * s.uy;
+        s.pz += s_int * s.uz;
+        s.dsafe = s.dsafe > s_int ? s.dsafe - s_int : 0.f;
+        return 2;
+      }
+    } else if (s.it < 0) {  // from the star: the polar cell of the direction
+      const float mu = s.uz;
+      s.it = warp_last(0, M.nt, [&](int i) { return M.cf[i] >= mu; });
+    }
+    const RayCuts q = ray_cuts(s.ir, s.it, s.px, s.py, s.pz, s.ux, s.uy, s.uz);
+    const int n_in = __popc(__ballot_sync(full, inner_hit(M, q, lane)));
+    const unsigned rough = __ballot_sync(full, lane < n_in && !inner_precise(M, q, lane));
+    const int n_ok = rough ? __ffs(rough) - 1 : 32;  // sphere crossings that count in this pass
+    const int n1 = __popc(__ballot_sync(full, cone_hit(M, q, lane)));
+    const bool cones = meets_cones(q, n1);
+    const float sr = sphere_cut(M, q, n_in, lane), st = cones ? cone_cut(M, q, n1, lane) : inf_<float>();
+    // lane m: i sphere and j = m - i cone crossings before its cell
+    int i = lane, j = 0;
+    float start = __shfl_up_sync(full, sr, 1), end = sr;
+    bool radial = true;  // the crossing into the lane's cell
+    if (lane == 0) start = 0.f;
+    if (cones) {
+      int hi = lane;
+      i = 0;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int mid = (i + hi) >> 1;
+        const int o = lane - 1 - mid;
+        const float a = __shfl_sync(full, sr, mid), c = __shfl_sync(full, st, o > 0 ? o : 0);
+        if (i < hi) {
+          if (a < c) i = mid + 1;
+          else hi = mid;
+        }
+      }
+      j = lane - i;
+      float a = __shfl_sync(full, sr, i > 0 ? i - 1 : 0), c = __shfl_sync(full, st, j > 0 ? j - 1 : 0);
+      end = fminf(__shfl_sync(full, sr, i), __shfl_sync(full, st, j));
+      if (i == 0) a = 0.f;
+      if (j == 0) c = 0.f;
+      radial = j == 0 || (i > 0 && a >= c);
+      start = fmaxf(a, c);
+    }
+    int ir, it;
+    cut_cell(q, n_in, n1, i, j, ir, it);
+    const bool counts = i < n_ok && lane < 31;  // (lane 31 is where a pass without an end stops)
+    const bool inside = ir >= 0 && ir < M.nr && it >= 0 && it < M.nt;
+    const int cell = ir * M.nt + it;
+    const float alpha = inside ? ldg(M.rho + cell) * chi : 0.f;
+    float x, y, z;
+    const float corr = entry_point(M, q, n_in, n1, i, j, radial, start, x, y, z);
+    const float len = fmaxf(end - start, 0.f);
+    float cum = inside && counts ? alpha * len : 0.f;  // optical depth up to the end of the lane's cell
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float v = __shfl_up_sync(full, cum, o);
+      if (lane >= o) cum += v;
+    }
+    // (a pass that ends in the lane's cell has gone the entry's correction further in the one before)
+    float before = __shfl_up_sync(full, cum, 1) + corr * __shfl_up_sync(full, alpha, 1);
+    if (lane == 0) before = 0.f;
+    const unsigned hits = __ballot_sync(full, inside && counts && cum > s.tau);
+    const unsigned outs = __ballot_sync(full, ir >= M.nr);
+    const unsigned cav = __ballot_sync(full, ir < 0);
+    const int n = __ffs(hits | outs | __ballot_sync(full, !counts)) - 1;  // crossings made in this pass
+    const bool hit = (hits >> n) & 1u;  // (a cell with an interaction lies inside the grid)
+    // entries of the cells, path lengths of the flight in each
+    if (lane >= 1 && lane <= n && inside) atomicAdd(M.visits + cell, 1ull);
+    // from the cell's entry (the lane of the interaction)
+    const float s_hit = fminf(fmaxf((s.tau - before) / alpha, 0.f), len);
+    const float last = JT ? __shfl_down_sync(full, corr, 1) : 0.f;
+    if (JT && inside && alpha > 0.f) {
+      const float l = lane < n ? len + (lane == n - 1 ? last : 0.f) : (hit && lane == n ? s_hit : 0.f);
+      if (l > 0.f) atomicAdd(M.jlen + (size_t)cell * M.nlam + s.lam, (double)l);
+    }
+    // (polar cells are not counted inside the cavity)
+    const unsigned ncross = (unsigned)n - __popc(cav & (cav << 1) & ((2u << n) - 1u));
+    acc.cross += ncross;
+    s.steps += ncross;
+    s.xcross += ncross;
+    s.ir = __shfl_sync(full, ir, n);
+    s.it = __shfl_sync(full, it, n);
+    if (s.ir >= M.nr) {
+      if (P.want_lam) resolve_pending(M, s);
+      int ib = (int)(fabsf(s.uz) * (float)kNInc);
+      ib = ib < kNInc ? ib : kNInc - 1;
+      if (lane == 0) atomicAdd(M.sed + s.lam * kNInc + ib, 1ull);
+      acc.escaped++;
+      return 0;
+    }
+    s.it = s.it < 0 ? 0 : (s.it < M.nt ? s.it : M.nt - 1);
+    if (hit) {
+      x += s_hit * s.ux;
+      y += s_hit * s.uy;
+      z += s_hit * s.uz;
+    }
+    s.px = __shfl_sync(full, x, n);
+    s.py = __shfl_sync(full, y, n);
+    s.pz = __shfl_sync(full, z, n);
+    s.alpha = __shfl_sync(full, alpha, n);
+    s.ialpha = s.alpha > 0.f ? 1.f / s.alpha : 0.f;
+    s.dsafe = 0.f;
+    if (n > 0) s.ninc = 0;
+    if (hit) {
+      s.tau = 0.f;
+      s.xcross = 0;
+      return 2;
+    }
+    s.tau = fmaxf(s.tau - __shfl_sync(full, before, n), 0.f);
+    if (s.xcross > 100000u) {
+      acc.err |= kErrStepGuard;
+      acc.capped++;
+      note_trip<float, WarpRng>(P, M, s, 2u);
+      return 0;
+    }
+  }
+}
+
+// mrw_chain with the wavelength at once. A jump's energy and the next Eq. 11 test need the cell's tally;
+// after the first jump it is the one the last deposit left (its returned old value, waited for only where
+// the next test uses it), and the exit bin is drawn once, for the last jump (the others' bins fly nowhere).
+// t: the tally the interaction before the chain left, 0 if it deposited nothing.
+template <bool G, bool JT>
+__device__ __forceinline__ void mrw_chain_now(const KParams<float>& P, WarpRng& rng, const DevModel<float>& M,
+                                              Pkt<float>& s, int c, Acc& acc, unsigned long long t, int& k) {
+  const bool lead0 = (threadIdx.x & 31u) == 0u;
+  const float rho = M.rho[c];
+  if (t == 0ull) t = *(volatile unsigned long long*)(M.tally + c);
+  unsigned long long old = 0, du = 0;
+  bool jumped = false;
+  float ul = 0.f;
+  for (;;) {
+    if (s.events >= P.max_events) break;
+    const float dm = dmin_cell(M, s.ir, s.it, s.px, s.py, s.pz);
+    s.dsafe = dm * dsafe_margin<float>();
+    if (jumped) t = __shfl_sync(0xffffffffu, old, 0) + du;
+    float w = 0.f, chiR = M.chiR0, kb = M.kbar0;
+    if (!(G || M.gray) || JT) qpos_warp(M, t, c, k, k, w);
+    if (!(G || M.gray)) {
+      chiR = (1.f - w) * __ldg(M.chiR + k) + w * __ldg(M.chiR + k + 1);
+      kb = (1.f - w) * __ldg(M.kbar + k) + w * __ldg(M.kbar + k + 1);
+    }
+    if (!(dm * rho * chiR > P.gamma)) break;  // Eq. 11
+    const uint4 ja = rng.next(s);  // escape-time quantile, point on the sphere, exit bin
+    const uint4 jb = rng.next(s);  // new direction
+    const float x = mrw_x(P, uni<float>(ja.x));
+    const float tau0 = dm * rho;
+    const float E = 3.f * x * tau0 * tau0 * chiR * kb;  // Eq. 9, as mrw_chain
+    float units = floorf(E * (float)kEUnit + 0.5f);
+    if (!(units < 1.8e19f)) {
+      units = 1.8e19f;
+      acc.err |= kErrMrwClip;
+    }
+    du = (unsigned long long)units;
+    if (lead0) old = atomicAdd(M.tally + c, du);
+    if (JT) j_walk<float, WarpRng>(M, c, 3.f * x * dm * dm * rho * chiR, k, w);
+    add_deposit(acc, du);
+    float hx, hy, hz;
+    iso_dir<float>(ja.y, ja.z, hx, hy, hz);
+    s.px += dm * hx;
+    s.py += dm * hy;
+    s.pz += dm * hz;
+    if (P.exit_dir == 1) {
+      s.ux = hx;
+      s.uy = hy;
+      s.uz = hz;
+      turn<float>(s.ux, s.uy, s.uz, sqrtf(uni<float>(jb.x)), uni<float>(jb.y));
+    } else {
+      iso_dir<float>(jb.x, jb.y, s.ux, s.uy, s.uz);
+    }
+    ul = uni<float>(ja.w);
+    s.events++;
+    acc.mrw++;
+    s.dsafe = 0.f;
+    jumped = true;
+  }
+  if (jumped && P.want_lam) {
+    t = __shfl_sync(0xffffffffu, old, 0) + du;
+    float w;
+    qpos_warp(M, t, c, k, k, w);
+    s.lam = sample_exit_warp(M, k, w, ul);
+    s.pend_mode = 0;
+    if (!(G || M.gray)) set_alpha<float, G>(M, s);
+  }
+}
+
+// interact with the wavelength at once; false: capped. kq: the T-grid interval of the packet's last
+// absorption (where the next one most likely lies)
+template <bool G, bool JT>
+__device__ __forceinline__ bool interact_now(const KParams<float>& P, WarpRng& rng, const DevModel<float>& M,
+                                             Pkt<float>& s, Acc& acc, bool release, int& kq) {
+  const int c = s.ir * M.nt + s.it;
+  const uint4 v = rng.next(s);  // albedo test, new direction, next optical depth
+  const float om = release ? 0.f : ((G || M.gray) ? M.alb0 : M.alb[s.lam]);
+  const float a = uni<float>(v.x);
+  const bool sca = a < om;
+  unsigned long long old = 0, left = 0;
+  if (!sca && (threadIdx.x & 31u) == 0u) {
+    old = atomicAdd(M.tally + c, kEUnit);
+    atomicAdd(M.nabs + c, 1ull);
+  }
+  const float g = sca ? ((G || M.gray) ? M.g0 : M.gq[s.lam]) : 0.f;
+  const float tau_next = neg_log<float>(uni<float>(v.w));
+  if (g != 0.f) turn<float>(s.ux, s.uy, s.uz, hg_mu(g, uni<float>(v.y)), uni<float>(v.z));
+  else iso_dir<float>(v.y, v.z, s.ux, s.uy, s.uz);
+  if (!sca) {
+    add_deposit(acc, kEUnit);
+    acc.abs++;
+    if (P.want_lam) {
+      old = __shfl_sync(0xffffffffu, old, 0);
+      left = old + kEUnit;
+      int ko;
+      float wo, wn;
+      qpos_warp(M, old, c, kq, ko, wo);
+      qpos_warp(M, left, c, ko, kq, wn);
+      s.lam = sample_bw_warp(M, ko, wo, kq, wn, (a - om) / (1.f - om));
+      s.pend_mode = 0;
+      if (!(G || M.gray)) set_alpha<float, G>(M, s);
+    }
+  } else {
+    acc.sca++;
+  }
+  s.events++;
+  s.ninc++;
+  if (P.mrw && s.ninc >= P.nmin) mrw_chain_now<G, JT>(P, rng, M, s, c, acc, left, kq);
+  if (s.events >= P.max_events) {
+    acc.capped++;
+    return false;
+  }
+  s.tau = tau_next;
+  return true;
+}
+
+// Runs a packet to its end, all 32 lanes carrying it: gray isotropic FP32 dust in runs of interactions,
+// FP32 dust that needs the wavelength at once in whole flights, everything else (polarization, the FP64
+// debug path, which keeps the oracle's order of floating-point operations) step by step.
+template <class R, bool G, bool POL, bool JT>
+__device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rng, const DevModel<R>& M, Pkt<R>& s,
+                                                Acc& acc) {
+  bool ended = false;
+  int kq = 0;
+  for (;;) {
+    if constexpr (sizeof(R) == 4 && !POL) {
+      if (JT || !(G || M.gray)) {
+        const bool release = s.pend == 2;
+        const int r = s.pend ? 2 : fly_warp<G, JT>(P, M, s, acc);
+        s.pend = 0;
+        if (r == 0 || !interact_now<G, JT>(P, rng, M, s, acc, release, kq)) return;
+        continue;
+      }
+    }
+    if (!POL && !JT && (G || M.gray) && sizeof(R) == 4 && !s.pend && s.ir >= 0 && s.alpha > (R)0 && M.g0 == (R)0 &&
+        s.events + 33u < P.max_events && s.steps + 33u < P.max_steps) {
+      const bool moved = interactions_at_once<R, G>(P, rng, M, s, acc, ended);
+      if (ended) return;
+      if (moved) continue;
+    }
+    if (!step<R, false, G, POL, JT>(P, rng, M, s, acc)) return;
+  }
+}
+
 // Tail of a transport launch (single disk or batch). When the queue drains, the packets still in flight are mostly long
 // ones (a lane holds a long packet for long), and lanes of one warp that follow different branches
 // share its issue slots, so in the transport kernel a long packet would then advance at a fraction of
@@ -1472,24 +1825,62 @@ __global__ void __launch_bounds__(32, kTailBlocksPerSm) transport_tail_kernel(co
       }
     } else {
       // all 32 lanes carry the packet: the same arithmetic in every lane, the random blocks computed
-      // 32 at a time, side effects by lane 0; gray isotropic dust takes runs of interactions at once
+      // 32 at a time, side effects by lane 0
       WarpRng rng{{(uint32_t)P.seed, (uint32_t)(P.seed >> 32)}, s.blk - 32u, make_uint4(0u, 0u, 0u, 0u)};
-      bool ended = false;
-      for (;;) {
-        // (FP32 only: the FP64 debug path keeps the oracle's order of floating-point operations)
-        if (!POL && !JT && (G || M.gray) && sizeof(R) == 4 && !s.pend && s.ir >= 0 && s.alpha > (R)0 && M.g0 == (R)0 &&
-            s.events + 33u < P.max_events && s.steps + 33u < P.max_steps) {
-          const bool moved = interactions_at_once<R, G>(P, rng, M, s, acc, ended);
-          if (ended) break;
-          if (moved) continue;
-        }
-        if (!step<R, TRACE, G, POL, JT>(P, rng, M, s, acc)) break;
-      }
+      run_packet_warp<R, G, POL, JT>(P, rng, M, s, acc);
     }
     if (lane == 0) {
       note_end(s, acc);
       if (BATCH) flush(M, acc, false);  // counters of the packet's model
     }
+  }
+  if (!BATCH && lane == 0) flush(P.m0, acc, false);
+}
+
+// 32-thread blocks of the warp kernel resident per SM (its register budget: 65536 / (32 x 16))
+constexpr int kWarpBlocksPerSm = 16;
+
+// Transport with one packet per warp from its launch to its end (run_packet_warp), packets taken one by
+// one from the queue: non-gray runs and batches. Their packets in flight are few (n_total / 3000), so the
+// time is the serial chain of the packets, not throughput: in a lane of the transport kernel a packet
+// waited for its 31 divergent neighbours (2.3 us a step); alone in a warp it waits for nobody, its flights
+// cross up to 31 cells in about the latency of two crossings, and its table searches take two dependent
+// loads. Measured (reset, run, temperatures, spectrum): 100x60 non-gray disk, tau_mid 1e5, MRW, 1e6 packets
+// 894 -> 222 ms (of which ~150 ms are its longest packets, ~7e4 steps of 2 us); 40x30, tau_mid 1e3, 1e6 packets
+// 160 -> 14.4 ms; a batch of six disks, 1.2e6 packets, 265 -> 19.8 ms. At full occupancy (1e7 packets, 2432
+// warps) a step costs as much as in the transport kernel, so every non-gray run takes this kernel.
+template <bool BATCH, bool JT>
+__global__ void __launch_bounds__(32, kWarpBlocksPerSm) transport_warp_kernel(const KParams<float> P) {
+  const unsigned lane = threadIdx.x & 31u;
+  Acc acc = Acc{};
+  for (;;) {
+    unsigned long long q = 0;
+    if (lane == 0) q = atomicAdd(P.queue, 1ull);
+    q = __shfl_sync(0xffffffffu, q, 0);
+    if (q >= P.total) break;
+    int m = 0;
+    unsigned long long local = q;
+    if (BATCH) {
+      if (P.qmap) {
+        const unsigned long long e = __ldg(P.qmap + (q >> 5));
+        m = (int)(e >> 48);
+        local = (e & 0xffffffffffffull) + (q & 31ull);
+      } else {
+        m = find_model(P, q);
+        local = q - P.models[m].q_begin;
+      }
+    }
+    const DevModel<float>& M = BATCH ? P.models[m] : P.m0;
+    if (local >= M.n_packets) continue;  // a padding slot of an interleaved queue
+    WarpRng rng{{(uint32_t)P.seed, (uint32_t)(P.seed >> 32)}, 0u - 32u, make_uint4(0u, 0u, 0u, 0u)};
+    Pkt<float> s;
+    launch_packet<float, false, false, false, JT>(P, rng, M, s, M.first_id + local, -1, acc);
+    run_packet_warp<float, false, false, JT>(P, rng, M, s, acc);
+    if (lane == 0) {
+      note_end(s, acc);
+      if (BATCH) flush(M, acc, false);
+    }
+    if (BATCH) acc = Acc{};
   }
   if (!BATCH && lane == 0) flush(P.m0, acc, false);
 }

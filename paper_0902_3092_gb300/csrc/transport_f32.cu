@@ -21,7 +21,7 @@ cudaError_t launch_transport_tail<float>(const KParams<float>& P, bool trace, bo
   const int grid = sms * (warps_per_sm > 0 ? warps_per_sm : kTailBlocksPerSm);
   if (batch) transport_tail_kernel<float, false, false, true><<<grid, 32, 0, st>>>(P);
   else if (gray) transport_tail_kernel<float, false, true, false><<<grid, 32, 0, st>>>(P);
-  else transport_tail_kernel<float, false, false, false><<<grid, 32, 0, st>>>(P);
+  else return cudaErrorInvalidValue;  // (non-gray FP32 runs with a tail are launch_transport_warp's)
   return cudaGetLastError();
 }
 
@@ -32,6 +32,19 @@ int transport_blocks_per_sm<float>(bool trace, bool batch, bool gray, int block)
   if (batch) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_kernel<float, false, true, false>, block, 0);
   else if (gray) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_kernel<float, false, false, true>, block, 0);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_kernel<float, false, false, false>, block, 0);
+  return n;
+}
+
+cudaError_t launch_transport_warp(const KParams<float>& P, bool batch, int warps, cudaStream_t st) {
+  if (batch) transport_warp_kernel<true, false><<<warps, 32, 0, st>>>(P);
+  else transport_warp_kernel<false, false><<<warps, 32, 0, st>>>(P);
+  return cudaGetLastError();
+}
+
+int transport_warps_per_sm(bool batch) {
+  int n = 0;
+  if (batch) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_warp_kernel<true, false>, 32, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_warp_kernel<false, false>, 32, 0);
   return n;
 }
 
