@@ -50,6 +50,9 @@ struct KParams {
   // model's first packet of the chunk (slots past a model's last packet are padding); NULL: each model's
   // packets one range of the queue (q_begin)
   const unsigned long long* qmap;
+  // the packets whose first flight from the star k_star_flights() left unfinished, their number behind
+  // queue[1] (single gray FP32 disks; NULL: the queue counts the packets themselves)
+  const unsigned long long* list;
   uint64_t seed;
   unsigned long long max_events;
   unsigned long long max_steps;  // loop guard per packet
@@ -667,6 +670,26 @@ __device__ __forceinline__ void launch_packet(const KParams<R>& P, RNG& rng, con
   trace_ev<R, TRACE>(P, s, EV_LAUNCH, -1);
   s.tau = neg_log<R>(uni<R>(w.w));
   acc.packets++;
+}
+
+// Launches listed packet e (its number | shell << 32 | polar row << 48): at its first interaction point if the
+// shell is not the first one, else from the star like every packet (in the first shell, the disk's sharp inner
+// rim, the mean free path may be a few roundings of the position).
+__device__ __forceinline__ void launch_listed(const DevModel<float>& M, Pkt<float>& s, unsigned long long e) {
+  const int ir = (int)(e >> 32) & 0xffff;
+  if (ir == 0) return;
+  s.it = (int)(e >> 48);
+  s.ir = ir;
+  set_alpha<float, true>(M, s);
+  const float N = ldg(M.ncol + (size_t)s.it * (M.nr + 1) + ir);
+  const float in = fminf((s.tau - N * M.chi0) * s.ialpha, M.rf[ir + 1] - M.rf[ir]);
+  const float r = M.rf[ir] + fmaxf(in, 0.f);
+  s.px = r * s.ux;
+  s.py = r * s.uy;
+  s.pz = r * s.uz;
+  s.steps = (unsigned)ir + 2u;
+  s.tau = 0.f;
+  s.pend = 1;
 }
 
 // safety margin applied to d_min when it serves as the lower bound of the distance to the cell boundary
@@ -1775,7 +1798,8 @@ __device__ __forceinline__ bool interact_now(const KParams<float>& P, WarpRng& r
 // Runs a packet to its end, all 32 lanes carrying it: gray isotropic FP32 dust in runs of interactions and
 // whole flights, FP32 dust that needs the wavelength at once in whole flights, everything else (polarization, the FP64
 // debug path, which keeps the oracle's order of floating-point operations) step by step.
-template <class R, bool G, bool POL, bool JT>
+// FLY: gray runs without the MRW.
+template <class R, bool G, bool POL, bool JT, bool FLY = false>
 __device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rng, const DevModel<R>& M, Pkt<R>& s,
                                                 Acc& acc) {
   bool ended = false;
@@ -1790,12 +1814,12 @@ __device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rn
         continue;
       }
     }
-    if constexpr (sizeof(R) == 4 && !POL && !JT) {
+    if constexpr (FLY) {
       // A flight that has crossed two faces most likely crosses more (a packet on its way out crosses all
       // shells): made whole, 31 cells in about the time of one interactions_at_once() call, which makes one
-      // crossing. 40x40 tau_mid = 100 disk, 1e6 packets: 2.2 -> 1.4 ms for the whole run. (Deciding by the
-      // flight's length against the shell's width, two loads per call, cost the long packets of the tau_mid =
-      // 1e6 disk 3 %.)
+      // crossing. 40x40 tau_mid = 100 disk, 1e6 packets: 2.2 -> 1.4 ms for the whole run. Not with the MRW:
+      // the tail's time is then its longest packets', which interact after every crossing or two, and this
+      // test cost them 1 to 3 %.
       if (!s.pend && (s.ir < 0 || s.xcross >= 2u)) {
         if (fly_warp<G, JT>(P, M, s, acc) == 0) return;
         s.pend = 1;
@@ -1817,7 +1841,7 @@ __device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rn
 // its speed alone. The transport kernel therefore stores them (state unchanged, so the random stream
 // and the result are the same) and this kernel runs them one per warp: lane 0 of each 32-thread block
 // takes packets from the pool, those that had taken at least kTailLongSteps steps first.
-template <class R, bool TRACE, bool G, bool BATCH, bool POL = false, bool JT = false>
+template <class R, bool TRACE, bool G, bool BATCH, bool POL = false, bool JT = false, bool FLY = false>
 __global__ void __launch_bounds__(32, kTailBlocksPerSm) transport_tail_kernel(const KParams<R> P) {
   const unsigned lane = threadIdx.x & 31u;
   if (TRACE && lane != 0) return;  // the debug trace runs one lane per packet
@@ -1838,7 +1862,7 @@ __global__ void __launch_bounds__(32, kTailBlocksPerSm) transport_tail_kernel(co
       // all 32 lanes carry the packet: the same arithmetic in every lane, the random blocks computed
       // 32 at a time, side effects by lane 0
       WarpRng rng{{(uint32_t)P.seed, (uint32_t)(P.seed >> 32)}, s.blk - 32u, make_uint4(0u, 0u, 0u, 0u)};
-      run_packet_warp<R, G, POL, JT>(P, rng, M, s, acc);
+      run_packet_warp<R, G, POL, JT, FLY>(P, rng, M, s, acc);
     }
     if (lane == 0) {
       note_end(s, acc);
@@ -1908,7 +1932,8 @@ template <class R, bool TRACE, bool BATCH, bool G, bool POL, bool JT>
 __host__ __device__ constexpr bool kLaneChains() { return sizeof(R) == 4 && !TRACE && !BATCH && G && !POL && !JT; }
 
 // G: gray dust known at compile time (single-disk gray runs); otherwise M.gray is read at run time.
-template <class R, bool TRACE, bool BATCH, bool G, bool POL = false, bool JT = false>
+// LIST: the packets of k_star_flights()'s list (gray FP32 runs without the MRW).
+template <class R, bool TRACE, bool BATCH, bool G, bool POL = false, bool JT = false, bool LIST = false>
 __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kernel(const KParams<R> P) {
   Pkt<R> s;
   Acc acc = Acc{};
@@ -1917,6 +1942,7 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
   int model = 0;
   const unsigned lane = threadIdx.x & 31;
   int until_refill = 0;
+  const unsigned long long total = LIST ? P.queue[1] : P.total;
   for (;;) {
     if (--until_refill < 0) {
       until_refill = P.refill - 1;
@@ -1928,9 +1954,13 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
         base = __shfl_sync(0xffffffffu, base, leader);
         if (!active && !done) {
           const unsigned long long q = base + __popc(need & ((1u << lane) - 1u));
-          if (q < P.total) {
+          if (q < total) {
             int m = 0;
-            unsigned long long local = q;
+            unsigned long long local = q, entry = 0;
+            if constexpr (LIST) {
+              entry = __ldg(P.list + q);
+              local = (uint32_t)entry;
+            }
             if (BATCH) {
               if (P.qmap) {
                 const unsigned long long e = __ldg(P.qmap + (q >> 5));
@@ -1949,6 +1979,10 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
             if (local < M.n_packets) {  // (a padding slot of an interleaved queue launches nothing)
               const int tslot = (TRACE && local < (unsigned long long)P.trace_n) ? (int)local : -1;
               launch_packet<R, TRACE, G, POL, JT>(P, rng, M, s, M.first_id + local, tslot, acc);
+              if constexpr (LIST) {
+                acc.packets--;  // (counted by k_star_flights)
+                launch_listed(M, s, entry);
+              }
               active = true;
             }
           } else {
@@ -2005,7 +2039,7 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
             const bool release = s.pend == 2;
             s.pend = 0;
             interact<R, TRACE, G, POL, JT>(P, rng, M, s, acc, release, &tau_next);
-            chain = P.mrw && s.ninc >= P.nmin;
+            chain = !LIST && P.mrw && s.ninc >= P.nmin;
           }
           if (__any_sync(0xffffffffu, chain)) mrw_chains_lanes(P, rng.key, M, s, acc, chain);
           if (inter) {
