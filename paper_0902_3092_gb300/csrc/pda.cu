@@ -25,8 +25,9 @@
 #include <vector>
 
 #include "internal.h"
-#include "tables.h"
+#include "cgcluster.cuh"
 #include "planck.cuh"
+#include "tables.h"
 
 namespace mcrt {
 
@@ -53,6 +54,7 @@ struct PdaState {
   DBuf w, gl, gk;                     // adjoint weights / gradient outputs (device staging)
   int n_pda = 0;
   int max_inner_alloc = 0;
+  int box[4] = {0, 0, 0, 0};          // rows [0, 1) and columns [2, 3) that hold the PDA cells
 };
 
 void pda_free(PdaState* p) { delete p; }
@@ -627,6 +629,23 @@ static std::vector<int> active_tiles(const std::vector<signed char>& mask, int w
   return t;
 }
 
+// rows [0, 1) and columns [2, 3) of the smallest box around the PDA cells (empty: all zero)
+static void pda_box(const std::vector<signed char>& mask, int nt, int* box) {
+  const int nr = (int)mask.size() / nt;
+  box[0] = nr;
+  box[2] = nt;
+  box[1] = box[3] = 0;
+  for (int i = 0; i < nr; ++i)
+    for (int j = 0; j < nt; ++j)
+      if (mask[(size_t)i * nt + j] == 2) {
+        box[0] = std::min(box[0], i);
+        box[1] = std::max(box[1], i + 1);
+        box[2] = std::min(box[2], j);
+        box[3] = std::max(box[3], j + 1);
+      }
+  if (box[1] <= box[0]) box[0] = box[1] = box[2] = box[3] = 0;
+}
+
 static mcrt_status pda_alloc(mcrt_disk* d, int max_inner) {
   PdaState* P = d->pda;
   if (!P) {
@@ -765,11 +784,15 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
   double norm_b = -1.0, best = INFINITY;
   int total_iters = 0, stall = 0;
   constexpr int chunk = 32;
+  // a region whose box fits one cluster is solved by one launch per refinement step (cgcluster.cuh)
+  const CgBox box{nt, P->box[0], P->box[2], P->box[1] - P->box[0], P->box[3] - P->box[2], P->ar.as<float>(),
+                  P->at.as<float>(), P->rs.as<double>(), 0.0, y, tol2_in, o->max_inner, P->kctr.as<int>()};
+  const CgPlan plan = cg_plan(box.rows, box.w, o->max_inner);
   // the CG iterations of one chunk as a CUDA graph (the index of the iteration lives on the device);
   // without a graph (capture refused, e.g. on the legacy default stream) the kernels launch one by one
   int* kdev = P->kctr.as<int>();
   ChunkGraph cg;
-  cudaGraphExec_t chunk_exec = cg.build(st, chunk, [&](int j) {
+  cudaGraphExec_t chunk_exec = plan.nc ? nullptr : cg.build(st, chunk, [&](int j) {
     launch_cg_iteration(P, n, nt, tiles, r, pb[(j + 1) & 1], pb[j & 1], Ap, y, sc, kdev, 0, o->max_inner, tol2_in, ga,
                         gb, st);
     k_iter_next<<<1, 1, 0, st>>>(kdev);
@@ -779,8 +802,11 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
     k_resid64<<<sgrid(n), 256, 0, st>>>(nr, nt, mask, Cr, Ct, dis, x, b, P->rs.as<double>(), red, 4);
     d->launches++;
     double rn2 = 0.0;
+    int made = 0;  // iterations of the last cluster solve
     CK(cudaMemcpyAsync(&rn2, red + 4, 8, cudaMemcpyDeviceToHost, st), "copy");
+    if (plan.nc && outer > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
     CK(cudaStreamSynchronize(st), "synchronize");
+    total_iters += made;
     const double rn = std::sqrt(rn2);
     if (norm_b < 0) norm_b = rn;  // first residual: x = 0 on the PDA cells, so this is |S b_total|
     if (!(rn == rn)) return set_error(d, MCRT_ENOTCONV, "PDA residual is not finite");
@@ -798,6 +824,15 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
     }
     if (outer == o->max_outer) break;
     // inner FP32 CG on the unit-diagonal system
+    if (plan.nc) {
+      CgBox b1 = box;
+      b1.inv_scale = 1.0 / rn;
+      CK(cg_solve(b1, plan, st), "PDA cluster kernel");
+      k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, rn, x);
+      d->launches += 2;
+      CK(cudaGetLastError(), "PDA kernels");
+      continue;
+    }
     CK(cudaMemsetAsync(sc, 0, sizeof(double) * (2 * (size_t)o->max_inner + 8), st), "memset");
     k_start<<<sgrid(n), 256, 0, st>>>(n, mask, P->rs.as<double>(), 1.0 / rn, y, r, pb[1], pb[0], Ap, sc);
     d->launches++;
@@ -933,6 +968,7 @@ mcrt_status mcrt_solve_pda(mcrt_disk* d, const mcrt_pda_opts* o, int* out_n, int
   P->vec4 = nt % 4 == 0;  // 16-byte kernels on 128-cell tiles
   P->htiles = active_tiles(hmask, P->vec4 ? 128 : 32);
   P->ntiles = (int)P->htiles.size();
+  pda_box(hmask, nt, P->box);
   if (P->ntiles > 0)
     CK(cudaMemcpyAsync(P->tiles.p, P->htiles.data(), P->htiles.size() * sizeof(int), cudaMemcpyHostToDevice, st),
        "copy");
@@ -1045,6 +1081,24 @@ __global__ void k_static_dis(int nr, int nt, const signed char* mask, const doub
     atomicAdd(red + 3, 1.0);
   }
 }
+// smallest box around the unknown cells, as atomic maxima that start at zero: nr - first row, last row + 1,
+// nt - first column, last column + 1
+__global__ void k_static_box(int nr, int nt, const signed char* mask, int* box) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  int v[4] = {0, 0, 0, 0};
+  if (c < nr * nt && mask[c] == 2) {
+    const int i = c / nt, j = c - i * nt;
+    v[0] = nr - i;
+    v[1] = i + 1;
+    v[2] = nt - j;
+    v[3] = j + 1;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int m = __reduce_max_sync(0xffffffffu, v[k]);
+    if ((threadIdx.x & 31u) == 0u && m) atomicMax(box + k, m);
+  }
+}
 // |S b|^2 of the system: the scaled residual with every unknown (mask 2) cell at 0, so that only the fixed
 // (mask 1) neighbours contribute; the solve's tolerance is relative to it, as in mcrt_solve_pda
 __global__ void k_static_bnorm(int nr, int nt, const signed char* mask, const double* Cr, const double* Ct,
@@ -1127,13 +1181,20 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
   k_static_dis<<<nblk(n), 256, 0, st>>>(nr, nt, mask_dev, Cr_dev, Ct_dev, dis, red);
   k_scaled<<<nblk(n), 256, 0, st>>>(nr, nt, mask_dev, Cr_dev, Ct_dev, dis, ar, at);
   k_static_bnorm<<<sgrid(n), 256, 0, st>>>(nr, nt, mask_dev, Cr_dev, Ct_dev, dis, u_dev, red);
-  double red_h[6] = {0, 0, 0, 0, 0, 0};
+  k_static_box<<<nblk(n), 256, 0, st>>>(nr, nt, mask_dev, reinterpret_cast<int*>(red + 6));
+  double red_h[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   CK(cudaMemcpyAsync(red_h, red, sizeof(red_h), cudaMemcpyDeviceToHost, st), "copy");
   CK(cudaStreamSynchronize(st), "synchronize");
   CK(cudaGetLastError(), "PDA kernels");
   if (red_h[3] > 0) return set_error(nullptr, MCRT_EINVAL, "a PDA cell has no conducting face (singular system)");
   const double norm_b = std::sqrt(red_h[5]);  // |S b|: the tolerance does not depend on the starting guess
   const double tol2_in = o->inner_tol * o->inner_tol;
+  // the region's box in one cluster, one launch per refinement step (cgcluster.cuh), if it fits
+  int bx[4], *const kdev = reinterpret_cast<int*>(red + 8);
+  std::memcpy(bx, red_h + 6, sizeof(bx));
+  const CgBox box{nt, nr - bx[0], nt - bx[2], bx[0] + bx[1] - nr, bx[2] + bx[3] - nt, ar, at, rs, 0.0, y, tol2_in,
+                  o->max_inner, kdev};
+  const CgPlan plan = bx[1] ? cg_plan(box.rows, box.w, o->max_inner) : CgPlan();
   const int ntiles = (n + 31) / 32;  // every tile of the grid
   const int ga = tgrid(k_cg_a<kUA>, ntiles), gb = tgrid(k_cg_b<kUB>, ntiles);
   double best = INFINITY;
@@ -1144,8 +1205,11 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
     CK(cudaMemsetAsync(red + 4, 0, sizeof(double), st), "memset");
     k_resid64<<<sgrid(n), 256, 0, st>>>(nr, nt, mask_dev, Cr_dev, Ct_dev, dis, u_dev, nullptr, rs, red, 4);
     double rn2 = 0.0;
+    int made = 0;  // iterations of the last cluster solve
     CK(cudaMemcpyAsync(&rn2, red + 4, sizeof(double), cudaMemcpyDeviceToHost, st), "copy");
+    if (plan.nc && outer > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
     CK(cudaStreamSynchronize(st), "synchronize");
+    total_iters += made;
     const double rn = std::sqrt(rn2);
     if (!(rn == rn)) return set_error(nullptr, MCRT_ENOTCONV, "PDA residual is not finite");
     if (rn <= o->tol * norm_b || rn == 0.0) {
@@ -1160,6 +1224,14 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
       return MCRT_OK;
     }
     if (outer == o->max_outer) break;
+    if (plan.nc) {
+      CgBox b1 = box;
+      b1.inv_scale = 1.0 / rn;
+      CK(cg_solve(b1, plan, st), "PDA cluster kernel");
+      k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, rn, u_dev);
+      CK(cudaGetLastError(), "PDA kernels");
+      continue;
+    }
     CK(cudaMemsetAsync(sc, 0, sizeof(double) * kStaticSc, st), "memset");
     k_start<<<sgrid(n), 256, 0, st>>>(n, mask_dev, rs, 1.0 / rn, y, r, pb[1], pb[0], Ap, sc);
     int k = 0;
