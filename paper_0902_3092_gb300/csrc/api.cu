@@ -70,34 +70,98 @@ const float* mrw_table(int device, cudaError_t* err) {
 // ------------------------------------------------------------------------------------------------
 // Temperatures (a7): 4 pi m sum_b kappa_b Bbar_b(T) = L_abs, FP64
 // ------------------------------------------------------------------------------------------------
-__global__ void k_temperature(int n, const unsigned long long* __restrict__ tally, const double* __restrict__ mass,
-                              double lfac, int gray, double kabs0, int nlam, const double* __restrict__ lam_e,
-                              const double* __restrict__ kabs, const double* __restrict__ lQk,
-                              const double* __restrict__ slQ, int nT, double Tmin, double dlnT,
-                              double* __restrict__ T, double* __restrict__ relerr) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n) return;
+// the counting error of cell c's tally and its absorbed luminosity per mass (0: no temperature)
+__device__ __forceinline__ double cell_q(int c, const unsigned long long* tally, const double* mass, double lfac,
+                                         double* relerr) {
   const unsigned long long t = tally[c];
   const double neq = (double)t / (double)kEUnit;
   if (relerr) relerr[c] = t ? 0.25 / sqrt(neq) : (double)INFINITY;
   const double m = mass[c];
-  if (t == 0ull || !(m > 0.0)) {
-    T[c] = 0.0;
-    return;
+  return t == 0ull || !(m > 0.0) ? 0.0 : neq * lfac / m;
+}
+
+// gray dust: closed form, one thread per cell
+__global__ void k_temperature_gray(int n, const unsigned long long* __restrict__ tally, const double* __restrict__ mass,
+                                   double lfac, double kabs0, double* __restrict__ T, double* __restrict__ relerr) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  const double q = cell_q(c, tally, mass, lfac, relerr);
+  T[c] = q > 0.0 ? pow(q / (4.0 * MCRT_SIGMA * kabs0), 0.25) : 0.0;
+}
+
+// Non-gray dust: one warp per 8 cells. The tabulated T of the cells in 8 lanes, then cell by cell the bin integrals of
+// the Newton step with the lanes over the bins (a bin's short edge is its neighbour lane's long one). A thread per
+// cell summed its 100 bins one after another: FP64 latency with too few threads (6000 cells: 3.3 ms), and warps that
+// waited for their widest cell.
+constexpr int kTempCells = 8;
+__global__ void __launch_bounds__(128) k_temperature(int n, const unsigned long long* __restrict__ tally,
+                                                     const double* __restrict__ mass, double lfac, int nlam,
+                                                     const double* __restrict__ lam_e, const double* __restrict__ kabs,
+                                                     const double* __restrict__ lQk, const double* __restrict__ slQ, int nT,
+                                                     double Tmin, double dlnT, double* __restrict__ T,
+                                                     double* __restrict__ relerr) {
+  const unsigned full = 0xffffffffu;
+  const int lane = (int)(threadIdx.x & 31u);
+  const int c0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kTempCells;
+  if (c0 >= n) return;
+  double q = 0.0, x = 0.0;
+  if (lane < kTempCells && c0 + lane < n) {
+    q = cell_q(c0 + lane, tally, mass, lfac, relerr);
+    if (q > 0.0) x = temperature_guess(q, lQk, slQ, nT, Tmin, dlnT);
   }
-  const double q = neq * lfac / m;
-  T[c] = cell_temperature(q, gray, kabs0, nlam, lam_e, kabs, lQk, slQ, nT, Tmin, dlnT);
+  const double pref = 8.0 * kPi * kKB * kKB * kKB * kKB / (kH * kH * kH * kC * kC);
+  for (unsigned todo = __ballot_sync(full, q > 0.0); todo; todo &= todo - 1u) {
+    const int l = __ffs(todo) - 1;
+    const double qc = __shfl_sync(full, q, l);
+    double xc = __shfl_sync(full, x, l), lo = 0.0, hi = INFINITY;
+    for (int it = 0; it < 100; ++it) {
+      const double hx = kH * kC / (1e-4 * kKB * xc);
+      double s3 = 0.0, s4 = 0.0, g3p = 0.0, g4p = 0.0;  // sums over the bins of kappa dG3, kappa dG4
+      for (int b0 = 0; b0 < nlam; b0 += 32) {
+        const int b = b0 + lane;
+        double g3 = 0.0, g4 = 0.0;
+        if (b < nlam) tails(b + 1 == nlam ? 0.0 : hx / lam_e[b + 1], g3, g4);
+        double a3 = __shfl_up_sync(full, g3, 1), a4 = __shfl_up_sync(full, g4, 1);
+        if (lane == 0) {
+          a3 = g3p;
+          a4 = g4p;
+        }
+        if (b < nlam) {
+          s3 += kabs[b] * (g3 - a3);
+          s4 += kabs[b] * (g4 - a4);
+        }
+        g3p = __shfl_sync(full, g3, 31);
+        g4p = __shfl_sync(full, g4, 31);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        s3 += __shfl_xor_sync(full, s3, o);
+        s4 += __shfl_xor_sync(full, s4, o);
+      }
+      const double p3 = pref * xc * xc * xc;
+      double xn;
+      const bool done = newton_step(qc, p3 * xc * s3, p3 * s4, xc, lo, hi, xn);
+      xc = xn;
+      if (done) break;
+    }
+    if (lane == l) x = xc;
+  }
+  if (lane < kTempCells && c0 + lane < n) T[c0 + lane] = x;
 }
 
 mcrt_status compute_temperatures(mcrt_disk* d) {
   const int n = d->nr * d->nt;
   const double lfac = d->Lpkt() / (d->n_total > 0 ? d->n_total : 1.0);
-  const double dlnT = std::log(d->Tmax / d->Tmin) / (d->nT - 2);
-  k_temperature<<<(n + 255) / 256, 256, 0, d->stream>>>(
-      n, d->tally.as<unsigned long long>(), d->mass_d.as<double>(), lfac, d->gray ? 1 : 0, d->kabs[0], d->nlam,
-      d->lam_e_d.as<double>(), d->kabs_d.as<double>(), d->lQ64.as<double>(), d->slQ64.as<double>(), d->nT, d->Tmin,
-      dlnT,
-      d->T_mc.as<double>(), d->relerr.as<double>());
+  const unsigned long long* tally = d->tally.as<unsigned long long>();
+  if (d->gray) {
+    k_temperature_gray<<<(n + 255) / 256, 256, 0, d->stream>>>(n, tally, d->mass_d.as<double>(), lfac, d->kabs[0],
+                                                               d->T_mc.as<double>(), d->relerr.as<double>());
+  } else {
+    const double dlnT = std::log(d->Tmax / d->Tmin) / (d->nT - 2);
+    k_temperature<<<(n + 4 * kTempCells - 1) / (4 * kTempCells), 128, 0, d->stream>>>(
+        n, tally, d->mass_d.as<double>(), lfac, d->nlam, d->lam_e_d.as<double>(), d->kabs_d.as<double>(),
+        d->lQ64.as<double>(), d->slQ64.as<double>(), d->nT, d->Tmin, dlnT, d->T_mc.as<double>(), d->relerr.as<double>());
+  }
   d->launches++;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(d, e, "temperature kernel");

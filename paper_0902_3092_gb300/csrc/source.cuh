@@ -53,10 +53,8 @@ __global__ void k_source(int nc, int nlam, const double* __restrict__ T, const d
       if (t > 0.0) {
         // bin b spans lam_e[b] .. lam_e[b+1]; G3 at the short edge is 0 for the first bin (lambda -> 0),
         // at the long edge G3(0) for the last one (lambda -> infinity)
-        double g_short = 0.0, g_long, g4;
-        if (b > 0) tails(kH * kC / (lam_e[b] * 1e-4 * kKB * t), g_short, g4);
-        if (b + 1 == nlam) tails(0.0, g_long, g4);
-        else tails(kH * kC / (lam_e[b + 1] * 1e-4 * kKB * t), g_long, g4);
+        const double g_short = b > 0 ? tail3(kH * kC / (lam_e[b] * 1e-4 * kKB * t)) : 0.0;
+        const double g_long = tail3(b + 1 == nlam ? 0.0 : kH * kC / (lam_e[b + 1] * 1e-4 * kKB * t));
         v = pref3 * (g_long - g_short) * kabs[b] / chi[b];
       }
       if (jlen) v += alb[b] * (jfac * jlen[(size_t)c * nlam + b] / cell_volume(rf, cf, nt, c));

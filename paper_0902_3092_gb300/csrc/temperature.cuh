@@ -28,17 +28,11 @@ __host__ __device__ inline void q_sum(const double* lam_e, const double* kabs, i
   dQ = 4.0 * kPi * p4 * s4;
 }
 
-// T with Q(T) = q > 0: gray dust in closed form, otherwise bracketed Newton from a cubic Hermite guess on
-// the tabulated grid (lQk: log Q(T_k), slQ: d log Q / d log T at T_k, T_k = Tmin exp((k-1) dlnT), k >= 1)
-__host__ __device__ inline double cell_temperature(double q, int gray, double kabs0, int nlam, const double* lam_e,
-                                                   const double* kabs, const double* lQk, const double* slQ, int nT,
-                                                   double Tmin, double dlnT) {
-  if (gray) {
-    return pow(q / (4.0 * MCRT_SIGMA * kabs0), 0.25);
-  }
-  // initial guess from the log-spaced grid: log T as a cubic Hermite function of log Q between the two
-  // grid temperatures that bracket q (slopes d log T / d log Q from the table; beyond the grid Q ~ T^4),
-  // then bracketed Newton on the exact bin integrals (about two evaluations from this guess)
+// The T of the tabulated grid for Q(T) = q > 0 (lQk: log Q(T_k), slQ: d log Q / d log T at T_k, T_k = Tmin exp((k-1)
+// dlnT), k >= 1): log T as a cubic Hermite function of log Q between the two grid temperatures that bracket q
+// (slopes d log T / d log Q from the table; beyond the grid Q ~ T^4). Within 2e-11 of the root on the grid.
+__host__ __device__ inline double temperature_guess(double q, const double* lQk, const double* slQ, int nT, double Tmin,
+                                                    double dlnT) {
   const double lq = log(q);
   double Tk;
   if (lq < lQk[1]) {
@@ -61,27 +55,36 @@ __host__ __device__ inline double cell_temperature(double q, int gray, double ka
     }
     Tk = Tmin * exp(y);
   }
-  double lo = 0.0, hi = INFINITY;
-  double x = Tk;
+  return Tk;
+}
+
+// One Newton step of the bracketed search from x, with Q and dQ/dT there (lo, hi: the bracket). True: xn is the root
+// to rounding. Q is smooth and increasing in T, so a step of relative size s leaves a relative error of order s^2:
+// below 1e-8 the new point is the root (this also ends a guess that is the root already, where f may be 0 and the
+// step would not lie strictly inside the bracket).
+__host__ __device__ inline bool newton_step(double q, double Q, double dQ, double x, double& lo, double& hi, double& xn) {
+  const double f = Q - q;
+  if (f > 0) hi = x; else lo = x;
+  xn = x - f / dQ;
+  if (fabs(xn - x) <= 1e-8 * x) return true;
+  if (!(xn > lo && xn < hi)) xn = isinf(hi) ? 2.0 * x : 0.5 * (lo + hi);
+  return fabs(xn - x) <= 1e-15 * x;
+}
+
+// T with Q(T) = q > 0: gray dust in closed form, otherwise bracketed Newton from the tabulated grid's T
+__host__ __device__ inline double cell_temperature(double q, int gray, double kabs0, int nlam, const double* lam_e,
+                                                   const double* kabs, const double* lQk, const double* slQ, int nT,
+                                                   double Tmin, double dlnT) {
+  if (gray) {
+    return pow(q / (4.0 * MCRT_SIGMA * kabs0), 0.25);
+  }
+  double lo = 0.0, hi = INFINITY, x = temperature_guess(q, lQk, slQ, nT, Tmin, dlnT);
   for (int it = 0; it < 100; ++it) {
-    double Q, dQ;
+    double Q, dQ, xn;
     q_sum(lam_e, kabs, nlam, x, Q, dQ);
-    const double f = Q - q;
-    if (f > 0) hi = x; else lo = x;
-    double xn = x - f / dQ;
-    // Q is smooth and increasing in T, so a Newton step of relative size s leaves a relative error of
-    // order s^2: below 1e-8 the new point is the root to rounding (this also ends a guess that is the
-    // root already, where f may be 0 and the step would not lie strictly inside the bracket)
-    if (fabs(xn - x) <= 1e-8 * x) {
-      x = xn;
-      break;
-    }
-    if (!(xn > lo && xn < hi)) xn = isinf(hi) ? 2.0 * x : 0.5 * (lo + hi);
-    if (fabs(xn - x) <= 1e-15 * x) {
-      x = xn;
-      break;
-    }
+    const bool done = newton_step(q, Q, dQ, x, lo, hi, xn);
     x = xn;
+    if (done) break;
   }
   return x;
 }
