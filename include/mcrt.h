@@ -246,7 +246,7 @@ mcrt_status mcrt_pda_adjoint_dev(mcrt_disk *d, const double *w_dev, double *grad
 /* Vertical hydrostatic structure (Sect. 2.5, Eq. 20): dP/dz = -rho G M_star z / R^3 with P = k_B rho T /
  * (mu m_u), at fixed surface density, from the disk's last temperatures. Each radial shell is one
  * column (z = r_c cos theta_c, R = r_c sin theta_c at the cell centres; trapezoid rule in z from
- * theta = 0 to pi) and keeps its dust mass; cells without dust stay without dust. One GPU thread per
+ * theta = 0 to pi) and keeps its dust mass; cells without dust stay without dust. One warp per
  * shell, FP64. The paper iterates transport -> temperatures -> this density until the mean change of
  * the temperatures between two iterations is below 3 sigma of their Monte Carlo errors. */
 typedef struct {

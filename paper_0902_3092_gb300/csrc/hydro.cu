@@ -7,7 +7,9 @@
 // is integrated with the trapezoid rule between consecutive cell centres from theta = 0 to pi, so
 // rho_j is proportional to exp(Phi_j) / T_j; each shell keeps its dust mass, cells without dust stay
 // without dust, and temperatures below T_floor (cells no packet heated) are raised to it.
-// One thread per shell, FP64 (a shell is a sequential sweep of a few hundred cells).
+// One warp per shell, FP64: the lanes take the shell's cells side by side (hydro.cuh). A
+// thread per shell swept its cells one after another, a few hundred threads on the whole GPU bound by FP64 latency
+// (200x120: 0.78 ms per call, with four allocations and the shell masses summed on the host).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -21,14 +23,55 @@ namespace {
 
 constexpr double kG = 6.67430e-8;  // cm^3 g^-1 s^-2
 
-__global__ void k_hydro(int nr, int nt, const double* __restrict__ rf, const double* __restrict__ tf,
-                        const double* __restrict__ T, const double* __restrict__ rho_cur,
-                        const double* __restrict__ shell_mass, double GM, double mu, double T_floor,
-                        const double* __restrict__ relax, double* __restrict__ rho_out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+struct WarpLanes {
+  __device__ int lane() const { return (int)(threadIdx.x & 31u); }
+  __device__ int size() const { return 32; }
+  __device__ double below(double x, double carry) const {
+    const double v = __shfl_up_sync(0xffffffffu, x, 1);
+    return lane() == 0 ? carry : v;
+  }
+  // In the order of the cells, one addition after another: near the pole the terms are 1e7 times the
+  // potential differences that matter, so another order of the sum has other roundings (1e-9 of the density).
+  __device__ double upto(double x, double carry) const {
+    double mine = carry;
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+      carry += __shfl_sync(0xffffffffu, x, l);
+      if (lane() == l) mine = carry;
+    }
+    return mine;
+  }
+  __device__ double last(double x) const { return __shfl_sync(0xffffffffu, x, 31); }
+  __device__ double sum(double x) const {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  }
+  __device__ double max(double x) const {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+  }
+};
+
+// shell_mass NULL: each shell keeps the sum of its cells' masses
+__global__ void __launch_bounds__(64) k_hydro(int nr, int nt, const double* __restrict__ rf, const double* __restrict__ tf,
+                                              const double* __restrict__ T, const double* __restrict__ rho_cur,
+                                              const double* __restrict__ mass, const double* __restrict__ shell_mass,
+                                              double GM, double mu, double T_floor, const double* __restrict__ relax,
+                                              double* rho_out) {
+  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (i >= nr) return;
-  hydro_shell(i, nt, rf, tf, T, rho_cur, shell_mass, GM, mu, T_floor, rho_out);
-  if (relax) hydro_relax(i, nt, rf, tf, rho_cur, relax[i], shell_mass, rho_out);
+  const WarpLanes g;
+  double M = 0.0;
+  if (shell_mass) {
+    M = shell_mass[i];
+  } else {
+    for (int j = g.lane(); j < nt; j += 32) M += mass[(size_t)i * nt + j];
+    M = g.sum(M);
+  }
+  hydro_shell_group(g, i, nt, rf, tf, T, rho_cur, M, GM, mu, T_floor, rho_out);
+  if (relax) hydro_relax_group(g, i, nt, rf, tf, rho_cur, relax[i], M, rho_out);
 }
 
 }  // namespace
@@ -65,17 +108,10 @@ mcrt_status mcrt_hydrostatic_density(mcrt_disk* d, const mcrt_hydro_opts* o, dou
   if (o->which == MCRT_T_PDA && !d->have_pda) return set_error(d, MCRT_ESTATE, "no PDA solution");
   const int nr = d->nr, nt = d->nt;
   const size_t n = (size_t)nr * nt;
-  std::vector<double> M(nr, 0.0);
-  if (o->shell_mass_g) {
-    for (int i = 0; i < nr; ++i) {
+  if (o->shell_mass_g)
+    for (int i = 0; i < nr; ++i)
       if (!(o->shell_mass_g[i] >= 0 && std::isfinite(o->shell_mass_g[i])))
         return set_error(d, MCRT_EINVAL, "shell masses must be finite and >= 0");
-      M[i] = o->shell_mass_g[i];
-    }
-  } else {
-    for (int i = 0; i < nr; ++i)
-      for (int j = 0; j < nt; ++j) M[i] += d->mass[(size_t)i * nt + j];
-  }
   if (o->relax)
     for (int i = 0; i < nr; ++i)
       if (!(o->relax[i] > 0.0 && o->relax[i] <= 2.0)) return set_error(d, MCRT_EINVAL, "relax must be in (0, 2]");
@@ -84,26 +120,30 @@ mcrt_status mcrt_hydrostatic_density(mcrt_disk* d, const mcrt_hydro_opts* o, dou
     mcrt_status s = compute_temperatures(d);
     if (s != MCRT_OK) return s;
   }
-  DBuf rf, tf, Md, out, rl;
-  if (o->relax) {
-    CK(rl.alloc(nr * 8), "cudaMalloc");
-    CK(cudaMemcpyAsync(rl.p, o->relax, nr * 8, cudaMemcpyHostToDevice, d->stream), "copy");
-  }
-  CK(rf.alloc((nr + 1) * 8), "cudaMalloc");
-  CK(tf.alloc((nt + 1) * 8), "cudaMalloc");
-  CK(Md.alloc(nr * 8), "cudaMalloc");
-  CK(out.alloc(n * 8), "cudaMalloc");
   cudaStream_t st = d->stream;
-  CK(cudaMemcpyAsync(rf.p, d->rf.data(), (nr + 1) * 8, cudaMemcpyHostToDevice, st), "copy");
-  CK(cudaMemcpyAsync(tf.p, d->tf.data(), (nt + 1) * 8, cudaMemcpyHostToDevice, st), "copy");
-  CK(cudaMemcpyAsync(Md.p, M.data(), nr * 8, cudaMemcpyHostToDevice, st), "copy");
+  // workspace kept with the disk: its faces (cm), uploaded once, the optional per-shell inputs, the density
+  const size_t nf = (size_t)nr + 1 + nt + 1;
+  if (d->hydro.n < (nf + 2 * (size_t)nr + n) * 8) {
+    CK(d->hydro.alloc((nf + 2 * (size_t)nr + n) * 8), "cudaMalloc");
+    cudaError_t e = cudaMemcpyAsync(d->hydro.p, d->rf.data(), (nr + 1) * 8, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(d->hydro.as<double>() + nr + 1, d->tf.data(), (nt + 1) * 8, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) {
+      d->hydro.release();
+      return cuda_fail(d, e, "copy");
+    }
+  }
+  double *const rf = d->hydro.as<double>(), *const tf = rf + nr + 1, *const Md = rf + nf, *const rl = Md + nr,
+                *const out = rl + nr;
+  if (o->shell_mass_g) CK(cudaMemcpyAsync(Md, o->shell_mass_g, nr * 8, cudaMemcpyHostToDevice, st), "copy");
+  if (o->relax) CK(cudaMemcpyAsync(rl, o->relax, nr * 8, cudaMemcpyHostToDevice, st), "copy");
   const double* T = (o->which == MCRT_T_PDA ? d->T_pda : d->T_mc).as<double>();
-  k_hydro<<<(nr + 127) / 128, 128, 0, st>>>(nr, nt, rf.as<double>(), tf.as<double>(), T, d->rho_cgs_d.as<double>(),
-                                            Md.as<double>(), kG * o->M_star_g, o->mu, o->T_floor_K,
-                                            o->relax ? rl.as<double>() : nullptr, out.as<double>());
+  k_hydro<<<(nr + 1) / 2, 64, 0, st>>>(nr, nt, rf, tf, T, d->rho_cgs_d.as<double>(), d->mass_d.as<double>(),
+                                       o->shell_mass_g ? Md : nullptr, kG * o->M_star_g, o->mu, o->T_floor_K,
+                                       o->relax ? rl : nullptr, out);
   d->launches++;
   CK(cudaGetLastError(), "hydrostatic kernel");
-  CK(cudaMemcpyAsync(rho_out, out.p, n * 8, cudaMemcpyDeviceToHost, st), "copy");
+  CK(cudaMemcpyAsync(rho_out, out, n * 8, cudaMemcpyDeviceToHost, st), "copy");
   CK(cudaStreamSynchronize(st), "synchronize");
   return MCRT_OK;
 }

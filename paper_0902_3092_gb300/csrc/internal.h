@@ -114,6 +114,7 @@ struct mcrt_disk {
   mcrt::DBuf ncol, first, list;  // first flights: column sums, counts per (row, last shell), the packets that go on
   mcrt::DBuf pool, pool_ctr;  // packets in flight when the queue drains (one slot per thread of the launch)
   unsigned pool_cap = 0;
+  mcrt::DBuf hydro;  // workspace of the hydrostatic density
   // temperatures
   mcrt::DBuf T_mc, relerr, T_pda;
   bool have_T = false, have_pda = false;
