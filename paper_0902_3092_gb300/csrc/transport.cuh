@@ -757,6 +757,10 @@ __device__ __forceinline__ float dmin_faces(const CellFaces& f, float px, float 
 // jump after jump, and each jump's deposit (Eq. 9) is computed after the loop by the lane that holds its
 // first block. The draws and the arithmetic of each jump are mrw_chain's; the deposits of the jumps of
 // one window are one atomic.
+// JT: the walks' path lengths go to the mean-intensity tally, each spread with the weights of the cell's T-grid
+// position when it starts, i.e. after the deposits of the jumps before it; the window's walks are added
+// bin by bin, one atomic per bin, and the exit bin is drawn at once.
+template <bool JT = false>
 __device__ __forceinline__ void mrw_chain_warp(const KParams<float>& P, WarpRng& rng, const DevModel<float>& M,
                                                Pkt<float>& s, int c, Acc& acc) {
   const unsigned lane = threadIdx.x & 31u;
@@ -812,13 +816,53 @@ __device__ __forceinline__ void mrw_chain_warp(const KParams<float>& P, WarpRng&
     for (int o = 16; o > 0; o >>= 1) dep += __shfl_xor_sync(full, dep, o);
     if (__any_sync(full, clip)) acc.err |= kErrMrwClip;
     if (k > 0) {
-      if (lane == 0) atomicAdd(M.tally + c, dep);
+      unsigned long long old = 0ull;
+      if (lane == 0) {
+        if (JT) old = atomicAdd(M.tally + c, dep);
+        else atomicAdd(M.tally + c, dep);
+      }
       add_deposit(acc, dep);
       const int last = 2 * (k - 1);
+      if constexpr (JT) {
+        old = __shfl_sync(full, old, 0);
+        unsigned long long before = du;  // deposits up to and with the lane's jump
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned long long v = __shfl_up_sync(full, before, o);
+          if ((int)lane >= o) before += v;
+        }
+        before -= du;
+        const bool walk = (lane & 1u) == 0u && (int)lane < 2 * k;
+        int kq = 0;
+        float wq = 0.f;
+        if (walk) qpos(M, old + before, c, kq, wq);
+        const float ct = walk ? 3.f * x * mydm * mydm * rho * chiR : 0.f;  // c t = x R0^2 / D, as mrw_chain
+        double* dst = M.jlen + (size_t)c * M.nlam;
+        for (int b0 = 0; b0 < M.nlam; b0 += 32) {
+          const int b = b0 + (int)lane;
+          double sum = 0.0;
+          for (int j = 0; j < k; ++j) {
+            const int kj = __shfl_sync(full, kq, 2 * j);
+            const float wj = __shfl_sync(full, wq, 2 * j), cj = __shfl_sync(full, ct, 2 * j);
+            if (b < M.nlam) {
+              const float* w0 = M.jw + (size_t)kj * M.nlam + b;
+              sum += (double)cj * (double)((1.f - wj) * __ldg(w0) + wj * __ldg(w0 + M.nlam));
+            }
+          }
+          if (sum > 0.0) atomicAdd(dst + b, sum);
+        }
+        if (P.want_lam) {  // the exit bin of the last jump
+          int kn;
+          float wn;
+          qpos(M, old + dep, c, kn, wn);
+          s.lam = sample_exit(M, kn, wn, __shfl_sync(full, ul, last));
+          s.pend_mode = 0;
+        }
+      }
       s.ux = __shfl_sync(full, nx, last + 1);
       s.uy = __shfl_sync(full, ny, last + 1);
       s.uz = __shfl_sync(full, nz, last + 1);
-      if (P.want_lam) {  // the exit bin of the last jump, drawn at escape
+      if (!JT && P.want_lam) {  // the exit bin of the last jump, drawn at escape
         s.pend_mode = 2;
         s.pend_cell = c;
         s.pend_u = __shfl_sync(full, ul, last);
@@ -831,9 +875,9 @@ __device__ __forceinline__ void mrw_chain_warp(const KParams<float>& P, WarpRng&
 template <class R, bool TRACE, bool G, bool POL = false, bool JT = false, class RNG>
 __device__ __forceinline__ void mrw_chain(const KParams<R>& P, RNG& rng, const DevModel<R>& M, Pkt<R>& s, int c,
                                           Acc& acc) {
-  if constexpr (RNG::coop && sizeof(R) == 4 && !TRACE && !POL && !JT) {
+  if constexpr (RNG::coop && sizeof(R) == 4 && !TRACE && !POL) {
     if ((G || M.gray) && P.exit_dir == 0) {
-      mrw_chain_warp(P, rng, M, s, c, acc);
+      mrw_chain_warp<JT>(P, rng, M, s, c, acc);
       return;
     }
   }
@@ -1339,7 +1383,13 @@ constexpr unsigned kMinRun = 24u;
 // cell. False when the call did nothing (advance()'s guard on crossings is due; the caller then takes a
 // normal step); sets `ended` when the packet ended (its MRW chain reached the event cap, or the crossing
 // left the grid).
-template <class R, bool G>
+// JT: the flights' path lengths go to the mean-intensity tally, each in the bin of the last absorption before it: the
+// run's absorptions in the cell are one atomic, whose returned old value gives each its own T_old and T_new in
+// their order, and their bins are drawn side by side. (60x40 gray disk, tau_mid = 1e4, MRW, 1e6 packets, run and ray
+// trace with scattered light: 168 -> 48 ms with this and the chains; one event at a time waited for an atomic's
+// old value and three table searches at every absorption, 2.3 us a step of the tail's longest packet. The
+// 200x120 tau_mid = 1e6 disk: 2.4 -> 0.63 s.)
+template <class R, bool G, bool JT = false>
 __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRng& rng, const DevModel<R>& M, Pkt<R>& s,
                                                     Acc& acc, bool& ended) {
   const unsigned lane = threadIdx.x & 31u;
@@ -1413,6 +1463,7 @@ __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRn
     s.steps++;
     s.xcross++;
     s.dsafe = (R)0;
+    if (JT) j_flight<R, WarpRng>(M, c, s.lam, s_face);
     if (!cross_face<R, false, G, false, WarpRng>(P, M, s, acc, s_face, fc, s.alpha)) ended = true;
     return true;
   }
@@ -1422,14 +1473,29 @@ __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRn
   const unsigned done_mask = n == 32 ? full : ((1u << n) - 1u);
   const unsigned absm = __ballot_sync(full, !(a < om)) & done_mask;
   const int nabs = __popc(absm);
+  int lam_abs = 0;  // JT: bin of the re-emission, in the lanes that absorb
   if (nabs) {
     const unsigned long long dep = (unsigned long long)nabs * kEUnit;
+    unsigned long long old = 0ull;
     if (lane == 0) {
-      atomicAdd(M.tally + c, dep);
+      if (JT) old = atomicAdd(M.tally + c, dep);
+      else atomicAdd(M.tally + c, dep);
       atomicAdd(M.nabs + c, (unsigned long long)nabs);
     }
     add_deposit(acc, dep);
-    if (P.want_lam) {  // the bin of the last absorption's re-emission, drawn at escape
+    if constexpr (JT) {
+      if (P.want_lam) {
+        old = __shfl_sync(full, old, 0);
+        if ((absm >> lane) & 1u) {
+          old += (unsigned long long)__popc(absm & ((1u << lane) - 1u)) * kEUnit;
+          int ko, kn;
+          float wo, wn;
+          qpos(M, old, c, ko, wo);
+          qpos(M, old + kEUnit, c, kn, wn);
+          lam_abs = sample_bw(M, ko, wo, kn, wn, (float)((a - om) / ((R)1 - om)));
+        }
+      }
+    } else if (P.want_lam) {  // the bin of the last absorption's re-emission, drawn at escape
       const R al = __shfl_sync(full, a, 31 - __clz(absm));
       s.pend_mode = 1;
       s.pend_cell = c;
@@ -1438,6 +1504,16 @@ __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRn
   }
   acc.abs += nabs;
   acc.sca += n - nabs;
+  if constexpr (JT) {
+    // flight k in the bin of the last absorption before interaction k; the flight that leaves the cell too
+    const unsigned prior = absm & ((1u << lane) - 1u);
+    const int from = P.want_lam && prior ? 31 - __clz(prior) : (int)lane;
+    const int lk = __shfl_sync(full, lam_abs, from);
+    const int lam = P.want_lam && prior ? lk : s.lam;
+    const bool leaves = !mrws && h < (int)m && (int)lane == h;
+    if ((int)lane < n || leaves) atomicAdd(M.jlen + (size_t)c * M.nlam + lam, (double)(leaves ? sf : f));
+    if (P.want_lam && absm) s.lam = __shfl_sync(full, lam_abs, 31 - __clz(absm));
+  }
   // the packet after interaction n-1
   const int l = n - 1;
   s.px = __shfl_sync(full, qx, l);
@@ -1467,7 +1543,7 @@ __device__ __forceinline__ bool interactions_at_once(const KParams<R>& P, WarpRn
     return true;
   }
   if (mrws) {
-    mrw_chain<R, false, G>(P, rng, M, s, c, acc);
+    mrw_chain<R, false, G, false, JT>(P, rng, M, s, c, acc);
     if (s.events >= P.max_events) {
       acc.capped++;
       ended = true;
@@ -1798,13 +1874,25 @@ __device__ __forceinline__ bool interact_now(const KParams<float>& P, WarpRng& r
 // Runs a packet to its end, all 32 lanes carrying it: gray isotropic FP32 dust in runs of interactions and
 // whole flights, FP32 dust that needs the wavelength at once in whole flights, everything else (polarization, the FP64
 // debug path, which keeps the oracle's order of floating-point operations) step by step.
-// FLY: gray runs without the MRW.
+// FLY: gray runs without the MRW or with the mean-intensity tally.
 template <class R, bool G, bool POL, bool JT, bool FLY = false>
 __device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rng, const DevModel<R>& M, Pkt<R>& s,
                                                 Acc& acc) {
   bool ended = false;
   int kq = 0;
   for (;;) {
+    // A flight that has crossed two faces most likely crosses more (a packet on its way out crosses all
+    // shells): made whole, 31 cells in about the time of one interactions_at_once() call, which makes one
+    // crossing. 40x40 tau_mid = 100 disk, 1e6 packets: 2.2 -> 1.4 ms for the whole run. Not with the MRW (but for
+    // the mean-intensity tally): the tail's time is then its longest packets', which interact after every
+    // crossing or two, and this test cost them 1 to 3 %.
+    const bool whole = FLY && !s.pend && (s.ir < 0 || s.xcross >= 2u);
+    if (!POL && sizeof(R) == 4 && !whole && (G || M.gray) && !s.pend && s.ir >= 0 && s.alpha > (R)0 && M.g0 == (R)0 &&
+        (!JT || P.exit_dir == 0) && s.events + 33u < P.max_events && s.steps + 33u < P.max_steps) {
+      const bool moved = interactions_at_once<R, G, JT>(P, rng, M, s, acc, ended);
+      if (ended) return;
+      if (moved) continue;
+    }
     if constexpr (sizeof(R) == 4 && !POL) {
       if (JT || !(G || M.gray)) {
         const bool release = s.pend == 2;
@@ -1814,22 +1902,11 @@ __device__ __forceinline__ void run_packet_warp(const KParams<R>& P, WarpRng& rn
         continue;
       }
     }
-    if constexpr (FLY) {
-      // A flight that has crossed two faces most likely crosses more (a packet on its way out crosses all
-      // shells): made whole, 31 cells in about the time of one interactions_at_once() call, which makes one
-      // crossing. 40x40 tau_mid = 100 disk, 1e6 packets: 2.2 -> 1.4 ms for the whole run. Not with the MRW:
-      // the tail's time is then its longest packets', which interact after every crossing or two, and this
-      // test cost them 1 to 3 %.
-      if (!s.pend && (s.ir < 0 || s.xcross >= 2u)) {
+    if constexpr (FLY && !JT) {
+      if (whole) {
         if (fly_warp<G, JT>(P, M, s, acc) == 0) return;
         s.pend = 1;
       }
-    }
-    if (!POL && !JT && (G || M.gray) && sizeof(R) == 4 && !s.pend && s.ir >= 0 && s.alpha > (R)0 && M.g0 == (R)0 &&
-        s.events + 33u < P.max_events && s.steps + 33u < P.max_steps) {
-      const bool moved = interactions_at_once<R, G>(P, rng, M, s, acc, ended);
-      if (ended) return;
-      if (moved) continue;
     }
     if (!step<R, false, G, POL, JT>(P, rng, M, s, acc)) return;
   }
@@ -1910,7 +1987,7 @@ __global__ void __launch_bounds__(32, kWarpBlocksPerSm) transport_warp_kernel(co
     WarpRng rng{{(uint32_t)P.seed, (uint32_t)(P.seed >> 32)}, 0u - 32u, make_uint4(0u, 0u, 0u, 0u)};
     Pkt<float> s;
     launch_packet<float, false, false, false, JT>(P, rng, M, s, M.first_id + local, -1, acc);
-    run_packet_warp<float, false, false, JT>(P, rng, M, s, acc);
+    run_packet_warp<float, false, false, JT, true>(P, rng, M, s, acc);
     if (lane == 0) {
       note_end(s, acc);
       if (BATCH) flush(M, acc, false);
