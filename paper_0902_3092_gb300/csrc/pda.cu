@@ -12,7 +12,8 @@
 //
 // Solve: FP64 iterative refinement. Each outer step forms r = b - A u in FP64 and solves the
 // Jacobi-scaled system (S A S) y = S r / |S r| (unit diagonal) with a matrix-free FP32 conjugate
-// gradient; u += |S r| S y. Two kernels per CG iteration: (A) p = r + beta p_old and Ap for the own
+// gradient; u += |S r| S y. A region whose box fits one thread-block cluster: one launch per step (cgcluster.cuh). Else two
+// kernels per CG iteration: (A) p = r + beta p_old and Ap for the own
 // cell and its four neighbours (p recomputed for neighbours from r and p_old, so no extra sweep),
 // with a block-reduced p.Ap; (B) y, r updates with a block-reduced r.r. The scalars live in a device
 // array indexed by the iteration, so the host only reads back once per chunk of iterations.
@@ -241,6 +242,10 @@ __global__ void k_scaled(int nr, int nt, const signed char* mask, const double* 
 
 // --------------------------------------------------------------------------------------------- FP64
 // rs = S (b + sum_f C_f (x_nb - x_c)) on PDA cells; red[slot] += |rs|^2
+// The factor that takes an inner right-hand side to FP32: a power of two, so that the last bits of rn (its blocks' sums are
+// added in any order) do not reach the FP32 solve: the same system gives the same solution.
+static double residual_scale(double rn) { return std::ldexp(1.0, std::ilogb(rn)); }
+
 __global__ void k_resid64(int nr, int nt, const signed char* __restrict__ mask, const double* __restrict__ Cr,
                           const double* __restrict__ Ct, const double* __restrict__ dis, const double* __restrict__ x,
                           const double* __restrict__ b, double* __restrict__ rs, double* red, int slot) {
@@ -840,18 +845,19 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
       return MCRT_OK;
     }
     if (outer == o->max_outer) break;
+    const double scale = residual_scale(rn);
     // inner FP32 CG on the unit-diagonal system
     if (plan.nc) {
       CgBox b1 = box;
-      b1.inv_scale = 1.0 / rn;
+      b1.inv_scale = 1.0 / scale;
       CK(cg_solve(b1, plan, st), "PDA cluster kernel");
-      k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, rn, x);
+      k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, scale, x);
       d->launches += 2;
       CK(cudaGetLastError(), "PDA kernels");
       continue;
     }
     CK(cudaMemsetAsync(sc, 0, sizeof(double) * (2 * (size_t)o->max_inner + 8), st), "memset");
-    k_start<<<sgrid(n), 256, 0, st>>>(n, mask, P->rs.as<double>(), 1.0 / rn, y, r, pb[1], pb[0], Ap, sc);
+    k_start<<<sgrid(n), 256, 0, st>>>(n, mask, P->rs.as<double>(), 1.0 / scale, y, r, pb[1], pb[0], Ap, sc);
     d->launches++;
     int k = 0;
     bool conv = false;
@@ -890,7 +896,7 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
       }
     }
     if (!conv) total_iters += k;
-    k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, rn, x);
+    k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, scale, x);
     d->launches++;
     CK(cudaGetLastError(), "PDA kernels");
   }
@@ -1241,16 +1247,17 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
       return MCRT_OK;
     }
     if (outer == o->max_outer) break;
+    const double scale = residual_scale(rn);
     if (plan.nc) {
       CgBox b1 = box;
-      b1.inv_scale = 1.0 / rn;
+      b1.inv_scale = 1.0 / scale;
       CK(cg_solve(b1, plan, st), "PDA cluster kernel");
-      k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, rn, u_dev);
+      k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, scale, u_dev);
       CK(cudaGetLastError(), "PDA kernels");
       continue;
     }
     CK(cudaMemsetAsync(sc, 0, sizeof(double) * kStaticSc, st), "memset");
-    k_start<<<sgrid(n), 256, 0, st>>>(n, mask_dev, rs, 1.0 / rn, y, r, pb[1], pb[0], Ap, sc);
+    k_start<<<sgrid(n), 256, 0, st>>>(n, mask_dev, rs, 1.0 / scale, y, r, pb[1], pb[0], Ap, sc);
     int k = 0;
     bool conv = false;
     while (k < o->max_inner && !conv) {
@@ -1278,7 +1285,7 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
       }
     }
     if (!conv) total_iters += k;
-    k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, rn, u_dev);
+    k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, scale, u_dev);
     CK(cudaGetLastError(), "PDA kernels");
   }
   if (out_iters) *out_iters = total_iters;
