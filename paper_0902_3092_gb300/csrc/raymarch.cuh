@@ -68,41 +68,58 @@ MCRT_HD int polar_index(const RayGrid<R>& G, R mu) {
   return lo;
 }
 
-// Calls emit(ir, it, L) for every cell the ray through sky point (p, q) crosses, in order of increasing
-// s (towards the observer), L the path length in the grid's length unit. (si, ci) = (sin i, cos i) of
-// the inclination the face table was built for. Returns the number of events, 0 if the ray misses the
-// grid, -1 if it took more than max_events.
-template <class R, class Emit>
-MCRT_HD int march_ray(const RayGrid<R>& G, R p, R q, R si, R ci, int max_events, Emit&& emit) {
-  using std::sqrt;
-  const R inf = (R)INFINITY;
-  const R b2 = p * p + q * q;
-  if (!(b2 < G.rf2[G.nr])) return 0;
-  const R z0 = q * si;
-  const R P1 = q * q * ci * ci + p * p;  // x0^2 + y0^2
-  const R P2 = z0 * z0;
-  const R Bq = -q * si * ci;
-  const R cb2 = ci * b2;
-  R s = -sqrt(G.rf2[G.nr] - b2);
-  R s0 = s;  // where the ray entered the current cell
-  int ir = G.nr - 1;
-  int it = polar_index(G, (z0 + s * ci) / sqrt(b2 + s * s));
-  // the polar angle falls (down) before the turning point s_e = cos(i) b^2 / z0 when z0 > 0 and after
-  // it when z0 < 0; the side is decided here and flipped at the turning point, never re-derived from
-  // the sign of cos(i) b^2 - z0 s near it, where rounding decides that sign
-  R se = inf;
-  bool turn = false, down;
-  if (z0 != (R)0) {
-    se = cb2 / z0;
-    turn = se > s;
-    down = turn ? z0 > (R)0 : z0 < (R)0;
-  } else {
-    down = cb2 > (R)0;
+// A ray on its way through the grid, an event (a face or the turning point of theta) at a time. (si, ci) = (sin i, cos i) of
+// the inclination the face table was built for.
+template <class R>
+struct RayMarch {
+  R si, ci, b2, z0, P1, P2, Bq, cb2;
+  R s, s0;      // now, and where the ray entered the current cell
+  R se;         // turning point of theta ahead
+  R sr, st;     // next radial and polar face
+  int ir, it, dr;
+  bool turn, down, need_r, need_t;
+
+  // false: the ray misses the grid
+  MCRT_HD bool begin(const RayGrid<R>& G, R p, R q, R si_, R ci_) {
+    using std::sqrt;
+    si = si_;
+    ci = ci_;
+    const R inf = (R)INFINITY;
+    b2 = p * p + q * q;
+    if (!(b2 < G.rf2[G.nr])) return false;
+    z0 = q * si;
+    P1 = q * q * ci * ci + p * p;  // x0^2 + y0^2
+    P2 = z0 * z0;
+    Bq = -q * si * ci;
+    cb2 = ci * b2;
+    s = -sqrt(G.rf2[G.nr] - b2);
+    s0 = s;
+    ir = G.nr - 1;
+    it = polar_index(G, (z0 + s * ci) / sqrt(b2 + s * s));
+    // the polar angle falls (down) before the turning point s_e = cos(i) b^2 / z0 when z0 > 0 and after
+    // it when z0 < 0; the side is decided here and flipped at the turning point, never re-derived from
+    // the sign of cos(i) b^2 - z0 s near it, where rounding decides that sign
+    se = inf;
+    turn = false;
+    if (z0 != (R)0) {
+      se = cb2 / z0;
+      turn = se > s;
+      down = turn ? z0 > (R)0 : z0 < (R)0;
+    } else {
+      down = cb2 > (R)0;
+    }
+    sr = inf;
+    st = inf;
+    dr = 1;
+    need_r = need_t = true;
+    return true;
   }
-  R sr = inf, st = inf;
-  int dr = 1;
-  bool need_r = true, need_t = true;
-  for (int n = 1; n <= max_events; ++n) {
+
+  // One event; emit(ir, it, L) if it ends a cell's segment. False: the ray has left the grid.
+  template <class Emit>
+  MCRT_HD bool step(const RayGrid<R>& G, Emit&& emit) {
+    using std::sqrt;
+    const R inf = (R)INFINITY;
     if (need_r) {  // radial face ahead
       if (s < (R)0 && G.rf2[ir] > b2) {
         sr = -sqrt(G.rf2[ir] - b2);
@@ -146,29 +163,40 @@ MCRT_HD int march_ray(const RayGrid<R>& G, R p, R q, R si, R ci, int max_events,
       turn = false;
       down = !down;
       need_t = true;
-      continue;
+      return true;
     }
-    if (st < sr) {
-      const R e = st > s ? st : s;
-      emit(ir, it, e - s0);
-      s = s0 = e;
+    const bool polar = st < sr;
+    const R x = polar ? st : sr;
+    const R e = x > s ? x : s;
+    emit(ir, it, e - s0);
+    s = s0 = e;
+    if (polar) {
       it += down ? -1 : 1;
       need_t = true;
-    } else {
-      const R e = sr > s ? sr : s;
-      emit(ir, it, e - s0);
-      s = s0 = e;
-      ir += dr;
-      need_r = true;
-      if (ir >= G.nr) return n;
-      if (ir < 0) {  // the cavity inside the inner radius: no dust, out at the far side of r_in
-        s = s0 = sqrt(G.rf2[0] - b2);
-        ir = 0;
-        it = polar_index(G, (z0 + s * ci) / sqrt(b2 + s * s));
-        need_t = true;
-      }
+      return true;
     }
+    ir += dr;
+    need_r = true;
+    if (ir >= G.nr) return false;
+    if (ir < 0) {  // the cavity inside the inner radius: no dust, out at the far side of r_in
+      s = s0 = sqrt(G.rf2[0] - b2);
+      ir = 0;
+      it = polar_index(G, (z0 + s * ci) / sqrt(b2 + s * s));
+      need_t = true;
+    }
+    return true;
   }
+};
+
+// Calls emit(ir, it, L) for every cell the ray through sky point (p, q) crosses, in order of increasing
+// s (towards the observer), L the path length in the grid's length unit. Returns the number of events, 0 if the ray
+// misses the grid, -1 if it took more than max_events.
+template <class R, class Emit>
+MCRT_HD int march_ray(const RayGrid<R>& G, R p, R q, R si, R ci, int max_events, Emit&& emit) {
+  RayMarch<R> m;
+  if (!m.begin(G, p, q, si, ci)) return 0;
+  for (int n = 1; n <= max_events; ++n)
+    if (!m.step(G, emit)) return n;
   return -1;
 }
 
