@@ -37,7 +37,7 @@ struct CgBox {
   const double* rs;    // scaled residual (whole grid)
   double inv_scale;    // right-hand side r = rs * inv_scale
   float* y;            // solution (whole grid, box cells written)
-  double tol2;         // stop at rr <= tol2 rr0
+  double tol2;         // stop at rr <= kCgStop tol2 rr0
   int max_iter;
   int* iters;          // out: iterations made
 };
@@ -130,13 +130,20 @@ __device__ __forceinline__ void cluster_sums(float* v, FloatPair* s, float (*wsu
   }
 }
 
+// The preconditioned iterations leave more of the error in the slow components than the tile kernels' at the same
+// residual, so they stop at a third of the residual asked for: a few more iterations instead of a larger error of the
+// whole solve. Relative error of the PDA temperatures against a 64-bit direct solve, tile kernels / 1 / 0.1 here:
+// 400x200 non-gray 1.3e-13 / 3.8e-13 / 2.5e-14, 300x160 gray 5.9e-14 / 7.3e-14 / 1.5e-14, 68x160 non-gray 7e-14 / 2e-13 /
+// 2e-14; time of the call 21.8 / 3.91 / 4.17 ms, 8.3 / 1.21 / 1.28, 11.9 / 0.96 / 0.97.
+constexpr double kCgStop = 0.1;
+
 // The scalars of an iteration from r.z, z.Az and r.r (the same in every thread).
 struct CgScalars {
   float alpha = 0.f, beta = 0.f, rr_stop, pap = 0.f;
   FloatPair rz_old;
   bool first = true;
   __device__ CgScalars(FloatPair rz, FloatPair rr, double tol2)
-      : rr_stop((float)(tol2 * ((double)rr.hi + (double)rr.lo))), rz_old(rz) {}
+      : rr_stop((float)(kCgStop * tol2 * ((double)rr.hi + (double)rr.lo))), rz_old(rz) {}
   // false: converged (or r.r is no number)
   __device__ __forceinline__ bool direction(FloatPair rz, FloatPair zaz, FloatPair rr) {
     if (!(rr.hi > rr_stop)) return false;
@@ -281,7 +288,7 @@ __global__ void __launch_bounds__(cg_threads(K), 1) k_cg_cluster(const CgBox B) 
 // lanes' affine maps by shuffle (their multipliers are constants, kept in shared memory), E more to add the carry;
 // no barrier. The two neighbour rows are solved here too. Odd E keeps the lanes' shared-memory accesses free of bank
 // conflicts (E = 2: two-way). An iteration costs 2.9 us against 2.1; whole solves, diagonal -> line: PDA of the 400x200
-// disk 5.25 -> 3.97 ms, of a 200x120 disk 1.19 -> 0.75, equal couplings 98x58 0.89 -> 0.85, 198x118 2.06 -> 1.83,
+// disk 5.25 -> 3.97 ms (at the full residual, kCgStop = 1, as the others), of a 200x120 disk 1.19 -> 0.75, equal couplings 98x58 0.89 -> 0.85, 198x118 2.06 -> 1.83,
 // 98x278 3.12 -> 2.44, 22x18 0.31 -> 0.33, 298x10 0.47 -> 0.53 (iterations of the diagonal one on strong couplings pay
 // for those two many times over).
 constexpr int kScan = 10;  // scan multipliers per row and lane: five steps forward, five backward
