@@ -168,7 +168,8 @@ __host__ __device__ __forceinline__ float entry_point(const DevModel<float>& M, 
   x = q.px + s * q.ux;
   y = q.py + s * q.uy;
   z = q.pz + s * q.uz;
-  if (i + j == 0) return 0.f;
+  // (a lane past the flight's last crossing, s infinite, has no face: its number lies outside the tables)
+  if (i + j == 0 || !(s < inf_<float>())) return 0.f;
   float d;
   if (radial) {
     const float c = x * x + y * y + z * z - M.rf2[sphere_face(q, n_in, i - 1)], b = x * q.ux + y * q.uy + z * q.uz;
