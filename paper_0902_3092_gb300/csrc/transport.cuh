@@ -587,6 +587,16 @@ __device__ __forceinline__ void resolve_pending(const DevModel<R>& M, Pkt<R>& s)
   s.pend_mode = 0;
 }
 
+// The tally of cell c at the moment. Other packets deposit in it meanwhile, and what a warp that carries one packet does next
+// (Eq. 11, table searches by its lanes) follows from it: one load for all its lanes, which else might part.
+template <class RNG, class R>
+__device__ __forceinline__ unsigned long long tally_now(const DevModel<R>& M, int c) {
+  unsigned long long t = 0;
+  if (lead<RNG>()) t = *(volatile unsigned long long*)(M.tally + c);
+  if (RNG::coop) t = __shfl_sync(0xffffffffu, t, 0);
+  return t;
+}
+
 // extinction per unit length of the packet's cell at its wavelength
 template <class R, bool G>
 __device__ __forceinline__ void set_alpha(const DevModel<R>& M, Pkt<R>& s) {
@@ -892,9 +902,9 @@ __device__ __forceinline__ void mrw_chain(const KParams<R>& P, RNG& rng, const D
     if (G || M.gray) {
       chiR = M.chiR0;
       kb = M.kbar0;
-      if (JT) qpos(M, *(volatile unsigned long long*)(M.tally + c), c, kq, wq);
+      if (JT) qpos(M, tally_now<RNG>(M, c), c, kq, wq);
     } else {
-      qpos(M, *(volatile unsigned long long*)(M.tally + c), c, kq, wq);
+      qpos(M, tally_now<RNG>(M, c), c, kq, wq);
       chiR = (R)((1.f - wq) * __ldg(M.chiR + kq) + wq * __ldg(M.chiR + kq + 1));
       kb = (R)((1.f - wq) * __ldg(M.kbar + kq) + wq * __ldg(M.kbar + kq + 1));
     }
@@ -1765,7 +1775,7 @@ __device__ __forceinline__ void mrw_chain_now(const KParams<float>& P, WarpRng& 
                                               Pkt<float>& s, int c, Acc& acc, unsigned long long t, int& k) {
   const bool lead0 = (threadIdx.x & 31u) == 0u;
   const float rho = M.rho[c];
-  if (t == 0ull) t = *(volatile unsigned long long*)(M.tally + c);
+  if (t == 0ull) t = tally_now<WarpRng>(M, c);
   unsigned long long old = 0, du = 0;
   bool jumped = false;
   float ul = 0.f;
