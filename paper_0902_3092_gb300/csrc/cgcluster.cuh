@@ -475,9 +475,14 @@ struct CgPlan {
   size_t smem = 0;
 };
 
-// the plan's launch on a stream; check: whether the device can hold its cluster, nothing launched
+// dynamic shared memory of a plan's kernel at most (227 KB less the kernel's own few hundred bytes)
+constexpr int kCgSmem = 220 * 1024;
+
+// the plan's launch on a stream; check: whether the device can hold its cluster, nothing launched. (A kernel's limit belongs
+// to the process, and threads plan and launch boxes of different sizes: it is always set to the same value, never to
+// the plan's own size, which would take it from another thread between its plan and its launch.)
 inline cudaError_t cg_launch(const CgPlan& L, const CgBox* B, cudaStream_t st, bool check) {
-  cudaError_t e = cudaFuncSetAttribute(L.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+  cudaError_t e = cudaFuncSetAttribute(L.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(L.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -499,7 +504,7 @@ inline cudaError_t cg_launch(const CgPlan& L, const CgBox* B, cudaStream_t st, b
   return cudaLaunchKernelEx(&cfg, L.kernel, *B);
 }
 inline bool cg_resident(const CgPlan& L) {
-  if (L.smem <= 220 * 1024 && cg_launch(L, nullptr, nullptr, true) == cudaSuccess) return true;
+  if (L.smem <= kCgSmem && cg_launch(L, nullptr, nullptr, true) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
 }
