@@ -318,8 +318,12 @@ int sm_count(int device) {
   return v > 0 ? v : 1;
 }
 
+constexpr size_t kRayFaces = 200 * 1024;  // bytes of the face table (and a value per bin) at most
+constexpr int kRaySmem = (int)kRayFaces + 16 * 1024;  // with the segments: a launch's shared memory at most
+
 template <class R>
 size_t ray_smem(int nt) {
+  static_assert(kRayBlock * kRaySegs<R> * sizeof(RaySeg<R>) <= 16 * 1024, "kRaySmem");
   return (size_t)kRayBlock * kRaySegs<R> * sizeof(RaySeg<R>) + (size_t)(nt + 1) * sizeof(FaceCoef<R>);
 }
 
@@ -329,8 +333,8 @@ cudaError_t launch_trace_nb(mcrt_disk* d, RayState* rs, const DevModel<R>& M, co
   const int max_events = 4 * (d->nr + d->nt) + 64;
   const double inv_l = 1.0 / d->l_unit;
   const size_t smem = ray_smem<R>(d->nt);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_raytrace<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) {  // (the limit belongs to the process: one value, which no thread's launch lowers for another's)
+    cudaError_t e = cudaFuncSetAttribute(k_raytrace<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRaySmem);
     if (e != cudaSuccess) return e;
   }
   // rays per warp: 32, fewer until 16 warps per SM have some (26,112 rays: 8 per warp 0.68 ms, 32 per warp 1.4)
@@ -411,7 +415,8 @@ mcrt_status trace_impl(mcrt_disk* d, int which) {
   if (rs->img.n < img_bytes) CK(rs->img.alloc(img_bytes), "cudaMalloc");
   CK(cudaMemsetAsync(rs->cnt.p, 0, 2 * sizeof(unsigned long long), d->stream), "memset");
   const int sms = sm_count(d->device);
-  if ((size_t)(d->nt + 1) * sizeof(FaceCoef<R>) + (size_t)nlam * sizeof(R) > 200 * 1024) return set_error(d, MCRT_EINVAL, "too many polar cells for the ray-tracing face table");
+  if ((size_t)(d->nt + 1) * sizeof(FaceCoef<R>) + (size_t)nlam * sizeof(R) > kRayFaces)
+    return set_error(d, MCRT_EINVAL, "too many polar cells for the ray-tracing face table");
   CK(launch_trace<R>(d, rs, model_of<R>(d), chi_of<R>(d), sms), "ray-trace kernel");
   d->launches++;
   rs->img_prec = prec;
