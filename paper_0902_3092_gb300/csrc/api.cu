@@ -214,7 +214,6 @@ static DevModel<R> make_model(const mcrt_disk* d, bool f64) {
   m.sf = (const R*)(f64 ? d->sf64.p : d->sf32.p);
   m.fk = (const signed char*)d->fk.p;
   m.rho = (const R*)(f64 ? d->rho64.p : d->rho32.p);
-  m.ncol = d->ncol.as<float>();
   m.chi = (const R*)(f64 ? d->chi64.p : d->chi32.p);
   m.alb = (const R*)(f64 ? d->alb64.p : d->alb32.p);
   m.gq = (const R*)(f64 ? d->g64.p : d->g32.p);
@@ -315,7 +314,6 @@ mcrt_status upload_density(mcrt_disk* d) {
   cudaError_t e = upload(d->rho32, cast_vec<float>(da.rhol));
   if (e == cudaSuccess) e = upload(d->rho64, da.rhol);
   if (e == cudaSuccess) e = upload(d->lqm, da.lqm);
-  if (e == cudaSuccess) e = upload(d->ncol, da.ncol);
   if (e == cudaSuccess) e = upload(d->mass_d, d->mass);
   if (e == cudaSuccess) e = upload(d->rho_cgs_d, d->rho);
   if (e != cudaSuccess) return cuda_fail(d, e, "upload");
@@ -477,7 +475,7 @@ mcrt_status mcrt_disk_create(const mcrt_grid* grid, const mcrt_star* star, int d
   if (e == cudaSuccess) e = d->visits.alloc(ncell * 8);
   if (e == cudaSuccess) e = d->nabs.alloc(ncell * 8);
   if (e == cudaSuccess) e = d->cnt.alloc((C_NCNT + kTripWords) * 8);  // run counters, then the guard record
-  if (e == cudaSuccess) e = d->queue.alloc(32);  // queue head, packets in the list, head of the first flights
+  if (e == cudaSuccess) e = d->queue.alloc(8);
   if (e == cudaSuccess) e = d->T_mc.alloc(ncell * 8);
   if (e == cudaSuccess) e = d->relerr.alloc(ncell * 8);
   if (e == cudaSuccess) e = d->T_pda.alloc(ncell * 8);
@@ -725,32 +723,6 @@ static int warp_grid(uint64_t n_packets, int sms, int warps_per_sm, uint64_t max
   return (int)std::max<uint64_t>(1, g);
 }
 
-// Runs whose first flights are found at once (see k_star_flights): gray plain Monte Carlo of a single FP32 disk
-// whose packets all start from the star (a list entry holds 16 bits of shell and of polar row), up to 12 packets
-// per lane the device holds (1.4e6). In longer runs the re-emission bins, drawn at escape, tell the changed
-// order of the packets' deposits more and more from the marches' (difference of the two escape spectra over that of
-// two runs of marches: 1.4 - 3 up to 1e6 packets, 3 - 3.3 at 2e6, 3.5 - 6 from 4e6 on; it stays 0.3 - 0.4 of
-// the spectrum's own Monte Carlo noise throughout).
-static bool first_flights(const mcrt_disk* d, uint64_t n_packets, uint64_t lanes, bool pol, bool jt, const mcrt_run_opts* o) {
-  return d->gray && !o->mrw && !pol && !jt && o->tail_warps_per_sm >= 0 && d->n_src == 0 && d->nr < 65535 &&
-         d->nt < 65536 && n_packets <= 12 * lanes;
-}
-
-// their buffers: the counts per (row, last shell), zero between runs, and the list of the packets that go on.
-// Without them (allocation failure) every packet marches from the star.
-static bool first_flight_buffers(mcrt_disk* d, uint64_t n_packets) {
-  const size_t counts = (size_t)d->nt * (d->nr + 1) * 8, list = n_packets * 8;
-  cudaError_t e = cudaSuccess;
-  if (d->first.n < counts) {
-    e = d->first.alloc(counts);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d->first.p, 0, counts, d->stream);
-    if (e != cudaSuccess) d->first.release();
-  }
-  if (e == cudaSuccess && d->list.n < list) e = d->list.alloc(list);
-  if (e != cudaSuccess) cudaGetLastError();
-  return e == cudaSuccess;
-}
-
 // Queue of a batch with non-gray dust: chunks of 32 slots of one model, ordered so that every model moves
 // through its packets at the same pace (chunk k of model m at (k + 1/2) / chunks_m, ties by model), so that
 // each model has the launch's share of its packets in flight (see MCRT_NONGRAY_IN_FLIGHT in mcrt.h).
@@ -792,7 +764,7 @@ static mcrt_status run_impl(mcrt_disk* d, uint64_t n_packets, uint64_t seed, uin
   if (jt && trace) return set_error(d, MCRT_EINVAL, "the mean-intensity tally has no event trace");
   if (jt && pol) return set_error(d, MCRT_EINVAL, "polarized transport does not keep the mean intensity");
   CK(cudaMemsetAsync(d->cnt.p, 0, (C_NCNT + kTripWords) * 8, d->stream), "memset");
-  CK(cudaMemsetAsync(d->queue.p, 0, 32, d->stream), "memset");
+  CK(cudaMemsetAsync(d->queue.p, 0, 8, d->stream), "memset");
   DBuf ttype, tcell, tlam, tpos, tn;
   if (trace) {
     const size_t m = (size_t)n_packets * trace_max;
@@ -854,16 +826,16 @@ static mcrt_status run_impl(mcrt_disk* d, uint64_t n_packets, uint64_t seed, uin
       KParams<float> P;
       std::memset(&P, 0, sizeof(P));
       fill_params(P, o, seed, tab);
-      P.queue = d->queue.as<unsigned long long>();
-      P.trip = d->cnt.as<unsigned long long>() + C_NCNT;
-      P.want_lam = (!d->gray || o->want_sed) ? 1 : 0;
-      const uint64_t cap = in_flight_cap(d->gray, d->n_total, o->max_in_flight);
       P.m0 = d->model32();
       P.m0.first_id = first_id;
       P.m0.n_packets = n_packets;
       P.m0.q_begin = 0;
       P.m0.model_id = 0;
       P.total = n_packets;
+      P.queue = d->queue.as<unsigned long long>();
+      P.trip = d->cnt.as<unsigned long long>() + C_NCNT;
+      P.want_lam = (!d->gray || o->want_sed) ? 1 : 0;
+      const uint64_t cap = in_flight_cap(d->gray, d->n_total, o->max_in_flight);
       if (one_packet_per_warp(d->gray, pol, o)) {
         const int warps = warp_grid(n_packets, dev_sms, jt ? transport_warps_per_sm_j() : transport_warps_per_sm(false), cap);
         e = jt ? launch_transport_warp_j(P, warps, d->stream) : launch_transport_warp(P, false, warps, d->stream);
@@ -874,20 +846,10 @@ static mcrt_status run_impl(mcrt_disk* d, uint64_t n_packets, uint64_t seed, uin
                              : transport_blocks_per_sm<float>(false, false, d->gray, block);
         const int grid = transport_grid(n_packets, block, dev_sms, bps, cap);
         const bool tail = setup_pool(d, P, (unsigned)grid * block, o->tail_warps_per_sm);
-        e = cudaSuccess;
-        if (first_flights(d, n_packets, (uint64_t)dev_sms * std::max(1, bps) * block, pol, jt, o) &&
-            first_flight_buffers(d, n_packets)) {
-          P.m0.first = d->first.as<unsigned long long>();
-          P.list = d->list.as<unsigned long long>();
-          e = launch_star_flights(P, d->list.as<unsigned long long>(), dev_sms, d->stream);
-          d->launches += 2;
-        }
-        if (e == cudaSuccess) {
-          e = pol  ? launch_transport_pol<float>(P, d->gray, grid, block, d->stream)
-              : jt ? launch_transport_j<float>(P, d->gray, grid, block, d->stream)
-                   : launch_transport<float>(P, false, false, d->gray, grid, block, d->stream);
-          d->launches++;
-        }
+        e = pol  ? launch_transport_pol<float>(P, d->gray, grid, block, d->stream)
+            : jt ? launch_transport_j<float>(P, d->gray, grid, block, d->stream)
+                 : launch_transport<float>(P, false, false, d->gray, grid, block, d->stream);
+        d->launches++;
         if (e == cudaSuccess && tail) {
           e = pol  ? launch_transport_tail_pol<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)
               : jt ? launch_transport_tail_j<float>(P, d->gray, dev_sms, o->tail_warps_per_sm, d->stream)

@@ -114,10 +114,6 @@ struct DevModel {
   const R* sf;            // nt+1 sin theta_f
   const signed char* fk;  // nt+1: +1 theta_f < pi/2, -1 theta_f > pi/2, 0 midplane plane, 2 axis
   const R* rho;           // nr*nt, rho * l_unit (g cm^-2)
-  // radial flights from the star (FP32): per polar row the column sum rho dr up to every radial face
-  // [nt][nr+1], and the packets whose first flight ended in shell k (nr: left the grid), [nt][nr+1]
-  const float* ncol;
-  unsigned long long* first;
   // dust per wavelength bin
   const R* chi;           // extinction kappa + sigma
   const R* alb;           // albedo sigma / chi

@@ -48,8 +48,6 @@ int transport_blocks_per_sm(bool trace, bool batch, bool gray, int block);
 template <class R>
 cudaError_t launch_transport_tail(const KParams<R>& P, bool trace, bool batch, bool gray, int sms, int warps_per_sm,
                                   cudaStream_t st);
-// the packets' first flights (FP32, single gray disk): fills `list` with the packets that go on, counts the rest
-cudaError_t launch_star_flights(const KParams<float>& P, unsigned long long* list, int sms, cudaStream_t st);
 // one packet per warp (FP32, non-gray runs and batches), `warps` warps in all: at most
 // transport_warps_per_sm per SM are resident
 cudaError_t launch_transport_warp(const KParams<float>& P, bool batch, int warps, cudaStream_t st);
@@ -111,7 +109,6 @@ struct mcrt_disk {
   mcrt::DBuf mass_d, rho_cgs_d;
   // tallies
   mcrt::DBuf tally, visits, nabs, sed, cnt, queue;
-  mcrt::DBuf ncol, first, list;  // first flights: column sums, counts per (row, last shell), the packets that go on
   mcrt::DBuf pool, pool_ctr;  // packets in flight when the queue drains (one slot per thread of the launch)
   unsigned pool_cap = 0;
   mcrt::DBuf hydro;  // workspace of the hydrostatic density

@@ -99,11 +99,10 @@ inline void geometry_arrays(int nr, int nt, const double* rf_cm, const double* t
 }
 
 // Density-dependent arrays: rho * l_unit (extinction per internal length unit per cm^2/g), the cell
-// masses (g) and log(1 / m) (FP32, 0 for empty cells), the radial column sums of every polar row (FP32 of FP64 sums).
+// masses (g) and log(1 / m) (FP32, 0 for empty cells).
 struct DensityArrays {
   std::vector<double> rhol, mass;
   std::vector<float> lqm;
-  std::vector<float> ncol;  // nt x (nr + 1): column sum rho * l_unit dr (dr in r_faces[0]) up to each radial face
 };
 inline void density_arrays(int nr, int nt, const double* rf_cm, const double* tf, const double* rho, DensityArrays& d) {
   const size_t ncell = (size_t)nr * nt;
@@ -119,15 +118,6 @@ inline void density_arrays(int nr, int nt, const double* rf_cm, const double* tf
       d.mass[c] = rho[c] * V;
       d.lqm[c] = d.mass[c] > 0 ? (float)(-std::log(d.mass[c])) : 0.f;
     }
-  d.ncol.resize((size_t)nt * (nr + 1));
-  for (int j = 0; j < nt; ++j) {
-    double sum = 0.0;
-    d.ncol[(size_t)j * (nr + 1)] = 0.f;
-    for (int i = 0; i < nr; ++i) {
-      sum += d.rhol[(size_t)i * nt + j] * ((rf_cm[i + 1] - rf_cm[i]) / rf_cm[0]);
-      d.ncol[(size_t)j * (nr + 1) + i + 1] = (float)sum;
-    }
-  }
 }
 
 // Dust per wavelength bin: extinction chi = kappa + sigma, albedo sigma / chi, chi' = kappa + (1 - g) sigma,

@@ -50,9 +50,6 @@ struct KParams {
   // model's first packet of the chunk (slots past a model's last packet are padding); NULL: each model's
   // packets one range of the queue (q_begin)
   const unsigned long long* qmap;
-  // the packets whose first flight from the star k_star_flights() left unfinished, their number behind
-  // queue[1] (single gray FP32 disks; NULL: the queue counts the packets themselves)
-  const unsigned long long* list;
   uint64_t seed;
   unsigned long long max_events;
   unsigned long long max_steps;  // loop guard per packet
@@ -680,26 +677,6 @@ __device__ __forceinline__ void launch_packet(const KParams<R>& P, RNG& rng, con
   trace_ev<R, TRACE>(P, s, EV_LAUNCH, -1);
   s.tau = neg_log<R>(uni<R>(w.w));
   acc.packets++;
-}
-
-// Launches listed packet e (its number | shell << 32 | polar row << 48): at its first interaction point if the
-// shell is not the first one, else from the star like every packet (in the first shell, the disk's sharp inner
-// rim, the mean free path may be a few roundings of the position).
-__device__ __forceinline__ void launch_listed(const DevModel<float>& M, Pkt<float>& s, unsigned long long e) {
-  const int ir = (int)(e >> 32) & 0xffff;
-  if (ir == 0) return;
-  s.it = (int)(e >> 48);
-  s.ir = ir;
-  set_alpha<float, true>(M, s);
-  const float N = ldg(M.ncol + (size_t)s.it * (M.nr + 1) + ir);
-  const float in = fminf((s.tau - N * M.chi0) * s.ialpha, M.rf[ir + 1] - M.rf[ir]);
-  const float r = M.rf[ir] + fmaxf(in, 0.f);
-  s.px = r * s.ux;
-  s.py = r * s.uy;
-  s.pz = r * s.uz;
-  s.steps = (unsigned)ir + 2u;
-  s.tau = 0.f;
-  s.pend = 1;
 }
 
 // safety margin applied to d_min when it serves as the lower bound of the distance to the cell boundary
@@ -2019,8 +1996,7 @@ template <class R, bool TRACE, bool BATCH, bool G, bool POL, bool JT>
 __host__ __device__ constexpr bool kLaneChains() { return sizeof(R) == 4 && !TRACE && !BATCH && G && !POL && !JT; }
 
 // G: gray dust known at compile time (single-disk gray runs); otherwise M.gray is read at run time.
-// LIST: the packets of k_star_flights()'s list (gray FP32 runs without the MRW).
-template <class R, bool TRACE, bool BATCH, bool G, bool POL = false, bool JT = false, bool LIST = false>
+template <class R, bool TRACE, bool BATCH, bool G, bool POL = false, bool JT = false>
 __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kernel(const KParams<R> P) {
   Pkt<R> s;
   Acc acc = Acc{};
@@ -2029,7 +2005,6 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
   int model = 0;
   const unsigned lane = threadIdx.x & 31;
   int until_refill = 0;
-  const unsigned long long total = LIST ? P.queue[1] : P.total;
   for (;;) {
     if (--until_refill < 0) {
       until_refill = P.refill - 1;
@@ -2041,13 +2016,9 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
         base = __shfl_sync(0xffffffffu, base, leader);
         if (!active && !done) {
           const unsigned long long q = base + __popc(need & ((1u << lane) - 1u));
-          if (q < total) {
+          if (q < P.total) {
             int m = 0;
-            unsigned long long local = q, entry = 0;
-            if constexpr (LIST) {
-              entry = __ldg(P.list + q);
-              local = (uint32_t)entry;
-            }
+            unsigned long long local = q;
             if (BATCH) {
               if (P.qmap) {
                 const unsigned long long e = __ldg(P.qmap + (q >> 5));
@@ -2066,10 +2037,6 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
             if (local < M.n_packets) {  // (a padding slot of an interleaved queue launches nothing)
               const int tslot = (TRACE && local < (unsigned long long)P.trace_n) ? (int)local : -1;
               launch_packet<R, TRACE, G, POL, JT>(P, rng, M, s, M.first_id + local, tslot, acc);
-              if constexpr (LIST) {
-                acc.packets--;  // (counted by k_star_flights)
-                launch_listed(M, s, entry);
-              }
               active = true;
             }
           } else {
@@ -2126,7 +2093,7 @@ __global__ void __launch_bounds__(256, transport_min_blocks<R>()) transport_kern
             const bool release = s.pend == 2;
             s.pend = 0;
             interact<R, TRACE, G, POL, JT>(P, rng, M, s, acc, release, &tau_next);
-            chain = !LIST && P.mrw && s.ninc >= P.nmin;
+            chain = P.mrw && s.ninc >= P.nmin;
           }
           if (__any_sync(0xffffffffu, chain)) mrw_chains_lanes(P, rng.key, M, s, acc, chain);
           if (inter) {

@@ -1,8 +1,5 @@
 // transport_f32.cu -- FP32 production instantiations of the transport kernel: single disk (gray dust
 // fixed at compile time, or not) and batches.
-#include <algorithm>
-
-#include "firstflight.cuh"
 #include "internal.h"
 
 namespace mcrt {
@@ -12,7 +9,6 @@ cudaError_t launch_transport<float>(const KParams<float>& P, bool trace, bool ba
                                     cudaStream_t st) {
   if (trace) return cudaErrorInvalidValue;
   if (batch) transport_kernel<float, false, true, false><<<grid, block, 0, st>>>(P);
-  else if (gray && P.list) transport_kernel<float, false, false, true, false, false, true><<<grid, block, 0, st>>>(P);
   else if (gray) transport_kernel<float, false, false, true><<<grid, block, 0, st>>>(P);
   else transport_kernel<float, false, false, false><<<grid, block, 0, st>>>(P);
   return cudaGetLastError();
@@ -38,19 +34,6 @@ int transport_blocks_per_sm<float>(bool trace, bool batch, bool gray, int block)
   else if (gray) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_kernel<float, false, false, true>, block, 0);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transport_kernel<float, false, false, false>, block, 0);
   return n;
-}
-
-cudaError_t launch_star_flights(const KParams<float>& P, unsigned long long* list, int sms, cudaStream_t st) {
-  const DevModel<float>& M = P.m0;
-  size_t smem = ((size_t)M.nlam * kNInc + M.nt) * sizeof(unsigned);
-  const int shared_rows = smem <= 48 * 1024;
-  if (!shared_rows) smem = (size_t)M.nlam * kNInc * sizeof(unsigned);  // (at most 1024 bins: 40 KB)
-  const int grid = (int)std::min<unsigned long long>((P.total + kStarBlock - 1) / kStarBlock, (unsigned long long)sms);
-  k_star_flights<<<grid, kStarBlock, smem, st>>>(P, list, shared_rows);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_first_visits<<<std::min((M.nt + 7) / 8, sms * 8), 256, 0, st>>>(M.nr, M.nt, M.first, M.visits);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_transport_warp(const KParams<float>& P, bool batch, int warps, cudaStream_t st) {
