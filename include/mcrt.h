@@ -100,7 +100,9 @@ mcrt_status mcrt_set_opacity(mcrt_disk *d, int nlam, const double *lam_edges_um,
  * the noise of its reference. So with non-gray dust and max_in_flight = 0, at most
  * n_total / MCRT_NONGRAY_IN_FLIGHT packets are in flight (at least one warp); gray dust, whose
  * trajectories no temperature changes, uses the whole device. Batches interleave their models' packets
- * so that each model keeps this share. */
+ * so that each model keeps this share. Where each packet has a warp (see mcrt_run_opts) and a disk's radial
+ * optical depth passes 2000 in some bin, a third of these are in flight: such packets' short ones pass the
+ * long ones faster, and the spectrum then stays as near to one packet after another. */
 #define MCRT_NONGRAY_IN_FLIGHT 3000
 
 typedef struct {
@@ -127,7 +129,8 @@ typedef struct {
   int interact_batch;           /* a warp runs the interaction code once this many of its lanes wait at
                                    an interaction point (or none can move on); 1: no waiting; 0: 8 */
   uint64_t max_in_flight;       /* at most this many packets in flight at once (the transport launch's
-                                   threads, rounded up to whole blocks); 0: one per thread the device
+                                   threads, rounded up to whole blocks; packets with a warp each: see
+                                   MCRT_NONGRAY_IN_FLIGHT); 0: one per thread the device
                                    holds for gray dust, n_total / MCRT_NONGRAY_IN_FLIGHT for non-gray
                                    dust (see there) */
 } mcrt_run_opts;

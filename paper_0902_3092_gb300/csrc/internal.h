@@ -81,6 +81,7 @@ struct mcrt_disk {
   double Tstar = 0, Rstar = 0, Lstar = 0;
   // internal sources (viscous heating): cumulative luminosity over the cells on the device, their total
   double Lsrc_total = 0;
+  double column = 0;  // largest radial column of the dust (g cm^-2)
   mcrt::DBuf src_cum;
   int n_src = 0;
   double Lpkt() const { return Lstar + Lsrc_total; }  // luminosity the packets carry

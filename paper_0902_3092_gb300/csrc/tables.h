@@ -99,16 +99,18 @@ inline void geometry_arrays(int nr, int nt, const double* rf_cm, const double* t
 }
 
 // Density-dependent arrays: rho * l_unit (extinction per internal length unit per cm^2/g), the cell
-// masses (g) and log(1 / m) (FP32, 0 for empty cells).
+// masses (g) and log(1 / m) (FP32, 0 for empty cells), the largest radial column rho dr (g cm^-2).
 struct DensityArrays {
   std::vector<double> rhol, mass;
   std::vector<float> lqm;
+  double column = 0.0;
 };
 inline void density_arrays(int nr, int nt, const double* rf_cm, const double* tf, const double* rho, DensityArrays& d) {
   const size_t ncell = (size_t)nr * nt;
   d.rhol.resize(ncell);
   d.mass.resize(ncell);
   d.lqm.resize(ncell);
+  std::vector<double> column(nt, 0.0);
   for (int i = 0; i < nr; ++i)
     for (int j = 0; j < nt; ++j) {
       const size_t c = (size_t)i * nt + j;
@@ -117,7 +119,9 @@ inline void density_arrays(int nr, int nt, const double* rf_cm, const double* tf
       const double V = 2.0 * kPi / 3.0 * (r2 * r2 * r2 - r1 * r1 * r1) * (std::cos(tf[j]) - std::cos(tf[j + 1]));
       d.mass[c] = rho[c] * V;
       d.lqm[c] = d.mass[c] > 0 ? (float)(-std::log(d.mass[c])) : 0.f;
+      column[j] += rho[c] * (r2 - r1);
     }
+  d.column = *std::max_element(column.begin(), column.end());
 }
 
 // Dust per wavelength bin: extinction chi = kappa + sigma, albedo sigma / chi, chi' = kappa + (1 - g) sigma,
