@@ -118,8 +118,11 @@ typedef struct {
                                    sources) / n_total);
                                    0 means the n_packets of this call */
   int block_size;               /* threads per block of the transport kernel (multiple of 32, <= 256);
-                                   0: tuned default (non-gray FP32 runs and batches with a tail carry one
-                                   packet per 32-thread block whatever the value) */
+                                   0: tuned default. FP32 runs and batches with non-gray dust and a tail carry
+                                   one packet per 32-thread block while at most 8 times the warps that the
+                                   device holds of them (16 per SM; 4 times with gray disks in the batch) are
+                                   allowed in flight; block_size, refill_interval, interact_batch and a
+                                   positive tail_warps_per_sm then mean nothing */
   int refill_interval;          /* steps between refills of finished lanes; 0: the default (8 for a single
                                    disk, tuned for a batch) */
   int want_sed;                 /* gray dust only: 0 skips the emission-bin sampling (no SED) */
@@ -175,7 +178,7 @@ mcrt_status mcrt_run_batch(mcrt_disk *const *disks, int n, const uint64_t *n_pac
 /* A prepared batch: many disks (uneven grids and packet budgets) transported by one persistent launch
  * over a shared packet queue, captured once as a CUDA graph and replayed. Disk i draws from the Philox
  * counter (block, model i, k), k = 0 .. n_packets[i]-1, and its packet energy is L_star / n_packets[i].
- * When opts->block_size == 0 a gray batch (or one without a tail) is autotuned on creation: block size
+ * When opts->block_size == 0 a batch with a packet per lane (see block_size) is autotuned on creation: block size
  * (64, 128, 256) and refill interval (1, 4, 16) are timed on a short run (about 5 % of the packets) and the
  * fastest is kept; with block_size == 0 the disks' tallies start from zero after the call. All disks must share one device;
  * the batch runs on the first disk's stream and must be destroyed before the disks. */

@@ -709,12 +709,23 @@ static uint64_t in_flight_cap(bool gray, double n_total, uint64_t requested) {
   return std::max<uint64_t>(32, (uint64_t)(n_total / MCRT_NONGRAY_IN_FLIGHT));
 }
 
-// Non-gray FP32 runs carry one packet per warp (transport_warp_kernel): few packets are in flight (see
-// MCRT_NONGRAY_IN_FLIGHT), so a packet that shares its warp with others only waits for them, and a warp's
-// lanes can take a flight's cells and a re-emission's table searches together. (tail_warps_per_sm = -1, the
-// form of the run whose packets all stay in the transport kernel, and polarized runs keep a packet per lane.)
-static bool one_packet_per_warp(bool gray, bool pol, const mcrt_run_opts* o) {
-  return !gray && !pol && o->tail_warps_per_sm >= 0;
+// Non-gray FP32 runs and batches carry one packet per warp (transport_warp_kernel) while the packets allowed in flight are up to
+// 8 times the warps that the device holds (16 per SM), batches with gray dust among them up to 4 times. Few packets are in
+// flight there (see MCRT_NONGRAY_IN_FLIGHT), so a packet that shares its warp with others only waits for them, and a warp's
+// lanes can take a flight's cells and a re-emission's table searches together. With more allowed, that many lanes do more
+// at once. 2432 warps, all that the device holds / lanes, by the packets allowed in flight:
+//   100x60, tau_mid 1e5   1e7 packets    6,000  319 / 668 ms    16,000  301 / 353    26,000  336 / 386    40,000  330 / 293
+//                         n / 3000 in flight, 3e7 packets  0.59 / 1.12 s    5e7  0.86 / 1.08    7e7  1.12 / 1.09    1e8  1.56 / 1.17
+//   40x30, tau_mid 1e3    1e7 packets    6,000   26 / 102 ms    16,000   26 / 38     20,000   26 / 31     26,000   26 / 25
+//                         3e7 packets       78 / 180 ms     5e7     129 / 181    7e7     181 / 186    1e8     258 / 194
+//   six such disks, 6e6 packets          6,000   21 / 64 ms     13,000   21 / 30     20,000   21 / 20     40,000   21 / 11
+//   one and five gray of 40x40, 6e6      6,000   32 / 63 ms     13,000   32 / 29     20,000   32 / 20     40,000   32 / 18
+// (tail_warps_per_sm = -1, the form of the run whose packets all stay in the transport kernel, and polarized runs keep a
+// packet per lane.)
+static bool one_packet_per_warp(bool gray, bool any_gray, bool pol, const mcrt_run_opts* o, uint64_t n_packets, uint64_t cap, int sms,
+                                int warps_per_sm) {
+  return !gray && !pol && o->tail_warps_per_sm >= 0 &&
+         std::min(n_packets, cap) <= (any_gray ? 4ull : 8ull) * sms * std::max(1, warps_per_sm);
 }
 
 // Warps of such a launch, one packet each: as many as a launch with a packet per lane may have packets in flight, a third of
@@ -856,9 +867,9 @@ static mcrt_status run_impl(mcrt_disk* d, uint64_t n_packets, uint64_t seed, uin
       P.trip = d->cnt.as<unsigned long long>() + C_NCNT;
       P.want_lam = (!d->gray || o->want_sed) ? 1 : 0;
       const uint64_t cap = in_flight_cap(d->gray, d->n_total, o->max_in_flight);
-      if (one_packet_per_warp(d->gray, pol, o)) {
-        const int warps = warp_grid(n_packets, dev_sms, jt ? transport_warps_per_sm_j() : transport_warps_per_sm(false), cap,
-                                    optically_thick(d));
+      const int held = jt ? transport_warps_per_sm_j() : transport_warps_per_sm(false);
+      if (one_packet_per_warp(d->gray, false, pol, o, n_packets, cap, dev_sms, held)) {
+        const int warps = warp_grid(n_packets, dev_sms, held, cap, optically_thick(d));
         e = jt ? launch_transport_warp_j(P, warps, d->stream) : launch_transport_warp(P, false, warps, d->stream);
         d->launches++;
       } else {
@@ -999,10 +1010,11 @@ mcrt_status mcrt_run_batch(mcrt_disk* const* disks, int n, const uint64_t* n_pac
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, d->device), "attribute");
   const int block = o->block_size ? o->block_size : 128;
   const uint64_t cap = in_flight_cap(!any_nongray, (double)q, o->max_in_flight);
-  const bool warp = one_packet_per_warp(!any_nongray, false, o);
-  bool thick = false;
-  for (int i = 0; i < n; ++i) thick |= optically_thick(disks[i]);
-  const int grid = warp ? warp_grid(P.total, dev_sms, transport_warps_per_sm(true), cap, thick)
+  bool thick = false, any_gray = false;
+  for (int i = 0; i < n; ++i) thick |= optically_thick(disks[i]), any_gray |= disks[i]->gray;
+  const int held = transport_warps_per_sm(true);
+  const bool warp = one_packet_per_warp(!any_nongray, any_gray, false, o, q, cap, dev_sms, held);
+  const int grid = warp ? warp_grid(q, dev_sms, held, cap, thick)
                         : transport_grid(P.total, block, dev_sms,
                                          transport_blocks_per_sm<float>(false, true, false, block), cap);
   cudaEvent_t ev0, ev1;
@@ -1430,7 +1442,10 @@ mcrt_status mcrt_batch_create(mcrt_disk* const* disks, int n, const uint64_t* n_
   auto grid_for = [&](int block) {
     return transport_grid(b->P.total, block, sms, transport_blocks_per_sm<float>(false, true, false, block), cap);
   };
-  b->warp = one_packet_per_warp(!any_nongray, false, o);
+  bool thick = false, any_gray = false;
+  for (int i = 0; i < n; ++i) thick |= optically_thick(disks[i]), any_gray |= disks[i]->gray;
+  const int held = transport_warps_per_sm(true);
+  b->warp = one_packet_per_warp(!any_nongray, any_gray, false, o, b->total, cap, sms, held);
   if (b->warp || o->block_size) {  // (one packet per warp: 32-thread blocks, nothing to tune)
     b->block = b->warp ? 32 : o->block_size;
     b->refill = o->refill_interval > 0 ? o->refill_interval : 1;
@@ -1495,9 +1510,7 @@ mcrt_status mcrt_batch_create(mcrt_disk* const* disks, int n, const uint64_t* n_
       }
     }
   b->P.refill = b->refill;
-  bool thick = false;
-  for (int i = 0; i < n; ++i) thick |= optically_thick(disks[i]);
-  b->grid = b->warp ? warp_grid(b->P.total, sms, transport_warps_per_sm(true), cap, thick) : grid_for(b->block);
+  b->grid = b->warp ? warp_grid(b->total, sms, held, cap, thick) : grid_for(b->block);
   // the tail kernel's pool: one slot per thread of the chosen launch (the autotuner ran without it)
   b->sms = sms;
   b->tail_warps = o->tail_warps_per_sm;

@@ -1946,8 +1946,8 @@ constexpr int kWarpBlocksPerSm = 16;
 // cross up to 31 cells in about the latency of two crossings, and its table searches take two dependent
 // loads. Measured (reset, run, temperatures, spectrum): 100x60 non-gray disk, tau_mid 1e5, MRW, 1e6 packets
 // 894 -> 222 ms (of which ~150 ms are its longest packets, ~7e4 steps of 2 us); 40x30, tau_mid 1e3, 1e6 packets
-// 160 -> 14.4 ms; a batch of six disks, 1.2e6 packets, 265 -> 19.8 ms. At full occupancy (1e7 packets, 2432
-// warps) a step costs as much as in the transport kernel, so every non-gray run takes this kernel.
+// 160 -> 14.4 ms; a batch of six disks, 1.2e6 packets, 265 -> 19.8 ms. Runs that may have many more
+// packets in flight than the device holds warps keep a packet per lane (see one_packet_per_warp).
 template <bool BATCH, bool JT>
 __global__ void __launch_bounds__(32, kWarpBlocksPerSm) transport_warp_kernel(const KParams<float> P) {
   const unsigned lane = threadIdx.x & 31u;

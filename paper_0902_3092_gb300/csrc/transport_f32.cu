@@ -22,7 +22,7 @@ cudaError_t launch_transport_tail<float>(const KParams<float>& P, bool trace, bo
   if (batch) transport_tail_kernel<float, false, false, true><<<grid, 32, 0, st>>>(P);
   else if (gray && !P.mrw) transport_tail_kernel<float, false, true, false, false, false, true><<<grid, 32, 0, st>>>(P);
   else if (gray) transport_tail_kernel<float, false, true, false><<<grid, 32, 0, st>>>(P);
-  else return cudaErrorInvalidValue;  // (non-gray FP32 runs with a tail are launch_transport_warp's)
+  else transport_tail_kernel<float, false, false, false><<<grid, 32, 0, st>>>(P);
   return cudaGetLastError();
 }
 
