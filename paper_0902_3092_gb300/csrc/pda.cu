@@ -651,23 +651,6 @@ static std::vector<int> active_tiles(const std::vector<signed char>& mask, int w
   return t;
 }
 
-// rows [0, 1) and columns [2, 3) of the smallest box around the PDA cells (empty: all zero)
-static void pda_box(const std::vector<signed char>& mask, int nt, int* box) {
-  const int nr = (int)mask.size() / nt;
-  box[0] = nr;
-  box[2] = nt;
-  box[1] = box[3] = 0;
-  for (int i = 0; i < nr; ++i)
-    for (int j = 0; j < nt; ++j)
-      if (mask[(size_t)i * nt + j] == 2) {
-        box[0] = std::min(box[0], i);
-        box[1] = std::max(box[1], i + 1);
-        box[2] = std::min(box[2], j);
-        box[3] = std::max(box[3], j + 1);
-      }
-  if (box[1] <= box[0]) box[0] = box[1] = box[2] = box[3] = 0;
-}
-
 static mcrt_status pda_alloc(mcrt_disk* d, int max_inner) {
   PdaState* P = d->pda;
   if (!P) {
@@ -991,7 +974,7 @@ mcrt_status mcrt_solve_pda(mcrt_disk* d, const mcrt_pda_opts* o, int* out_n, int
   P->vec4 = nt % 4 == 0;  // 16-byte kernels on 128-cell tiles
   P->htiles = active_tiles(hmask, P->vec4 ? 128 : 32);
   P->ntiles = (int)P->htiles.size();
-  pda_box(hmask, nt, P->box);
+  cg_box(hmask.data(), nr, nt, P->box);
   if (P->ntiles > 0)
     CK(cudaMemcpyAsync(P->tiles.p, P->htiles.data(), P->htiles.size() * sizeof(int), cudaMemcpyHostToDevice, st),
        "copy");

@@ -53,3 +53,9 @@ extern "C" int host_cg_solve(int rows, int w, int rows2, int w2) {
   fake::before_launch[0] = 0;
   return e == cudaSuccess ? 0 : 1;
 }
+
+// box of the cells with mask 2, and whether a box of its size has a plan
+extern "C" int host_cg_box(const signed char* mask, int nr, int nt, int* box) {
+  mcrt::cg_box(mask, nr, nt, box);
+  return mcrt::cg_plan(box[1] - box[0], box[3] - box[2], 1000).nc;
+}
