@@ -109,42 +109,10 @@ __global__ void __launch_bounds__(128) k_temperature(int n, const unsigned long 
     q = cell_q(c0 + lane, tally, mass, lfac, relerr);
     if (q > 0.0) x = temperature_guess(q, lQk, slQ, nT, Tmin, dlnT);
   }
-  const double pref = 8.0 * kPi * kKB * kKB * kKB * kKB / (kH * kH * kH * kC * kC);
   for (unsigned todo = __ballot_sync(full, q > 0.0); todo; todo &= todo - 1u) {
     const int l = __ffs(todo) - 1;
-    const double qc = __shfl_sync(full, q, l);
-    double xc = __shfl_sync(full, x, l), lo = 0.0, hi = INFINITY;
-    for (int it = 0; it < 100; ++it) {
-      const double hx = kH * kC / (1e-4 * kKB * xc);
-      double s3 = 0.0, s4 = 0.0, g3p = 0.0, g4p = 0.0;  // sums over the bins of kappa dG3, kappa dG4
-      for (int b0 = 0; b0 < nlam; b0 += 32) {
-        const int b = b0 + lane;
-        double g3 = 0.0, g4 = 0.0;
-        if (b < nlam) tails(b + 1 == nlam ? 0.0 : hx / lam_e[b + 1], g3, g4);
-        double a3 = __shfl_up_sync(full, g3, 1), a4 = __shfl_up_sync(full, g4, 1);
-        if (lane == 0) {
-          a3 = g3p;
-          a4 = g4p;
-        }
-        if (b < nlam) {
-          s3 += kabs[b] * (g3 - a3);
-          s4 += kabs[b] * (g4 - a4);
-        }
-        g3p = __shfl_sync(full, g3, 31);
-        g4p = __shfl_sync(full, g4, 31);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        s3 += __shfl_xor_sync(full, s3, o);
-        s4 += __shfl_xor_sync(full, s4, o);
-      }
-      const double p3 = pref * xc * xc * xc;
-      double xn;
-      const bool done = newton_step(qc, p3 * xc * s3, p3 * s4, xc, lo, hi, xn);
-      xc = xn;
-      if (done) break;
-    }
-    if (lane == l) x = xc;
+    const double root = temperature_root(WarpLanes(), __shfl_sync(full, q, l), __shfl_sync(full, x, l), nlam, lam_e, kabs);
+    if (lane == l) x = root;
   }
   if (lane < kTempCells && c0 + lane < n) T[c0 + lane] = x;
 }

@@ -23,37 +23,6 @@ namespace {
 
 constexpr double kG = 6.67430e-8;  // cm^3 g^-1 s^-2
 
-struct WarpLanes {
-  __device__ int lane() const { return (int)(threadIdx.x & 31u); }
-  __device__ int size() const { return 32; }
-  __device__ double below(double x, double carry) const {
-    const double v = __shfl_up_sync(0xffffffffu, x, 1);
-    return lane() == 0 ? carry : v;
-  }
-  // In the order of the cells, one addition after another: near the pole the terms are 1e7 times the
-  // potential differences that matter, so another order of the sum has other roundings (1e-9 of the density).
-  __device__ double upto(double x, double carry) const {
-    double mine = carry;
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      carry += __shfl_sync(0xffffffffu, x, l);
-      if (lane() == l) mine = carry;
-    }
-    return mine;
-  }
-  __device__ double last(double x) const { return __shfl_sync(0xffffffffu, x, 31); }
-  __device__ double sum(double x) const {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-  }
-  __device__ double max(double x) const {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-  }
-};
-
 // shell_mass NULL: each shell keeps the sum of its cells' masses
 __global__ void __launch_bounds__(64) k_hydro(int nr, int nt, const double* __restrict__ rf, const double* __restrict__ tf,
                                               const double* __restrict__ T, const double* __restrict__ rho_cur,

@@ -4,19 +4,9 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "lanes.cuh"
 
 namespace mcrt {
-
-// The threads that share a shell: one (the host), or a warp (the kernel), lane l taking the polar cells l, l + size, ...
-struct OneLane {
-  __host__ __device__ int lane() const { return 0; }
-  __host__ __device__ int size() const { return 1; }
-  __host__ __device__ double below(double, double carry) const { return carry; }   // the previous lane's x
-  __host__ __device__ double upto(double x, double carry) const { return carry + x; }  // carry + the lanes' sum so far
-  __host__ __device__ double last(double x) const { return x; }                      // the last lane's x
-  __host__ __device__ double sum(double x) const { return x; }
-  __host__ __device__ double max(double x) const { return x; }
-};
 
 // Shell i (cgs: rf, tf the grid faces, T the temperatures, rho_cur the current density, shell_mass its
 // mass): at the cell centres z = r_c cos theta_c, R = r_c sin theta_c, d ln(rho c^2)/dz = -G M z / (R^3 c^2)

@@ -152,26 +152,8 @@ __global__ void __launch_bounds__(128) k_kappaR(int nr, int nt, const signed cha
   }
   for (unsigned todo = __ballot_sync(full, Tc > 0.0); todo; todo &= todo - 1u) {
     const int l = __ffs(todo) - 1;
-    const double hx = kH * kC / (1e-4 * kKB * __shfl_sync(full, Tc, l));
-    double s1 = 0.0, s2 = 0.0, g4p = 0.0;
-    for (int b0 = 0; b0 < nlam; b0 += 32) {
-      const int b = b0 + lane;
-      double g3, g4 = 0.0;
-      if (b < nlam) tails(b + 1 == nlam ? 0.0 : hx / lam_e[b + 1], g3, g4);
-      double a4 = __shfl_up_sync(full, g4, 1);
-      if (lane == 0) a4 = g4p;
-      if (b < nlam) {
-        s1 += g4 - a4;
-        s2 += (g4 - a4) / chip[b];
-      }
-      g4p = __shfl_sync(full, g4, 31);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s1 += __shfl_xor_sync(full, s1, o);
-      s2 += __shfl_xor_sync(full, s2, o);
-    }
-    if (lane == l) k = s1 / s2;
+    const double mean = rosseland_group(WarpLanes(), lam_e, chip, nlam, __shfl_sync(full, Tc, l));
+    if (lane == l) k = mean;
   }
   if (c < n) kR[c] = k;
 }

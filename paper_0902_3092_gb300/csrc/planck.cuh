@@ -11,6 +11,8 @@
 #pragma once
 #include <cmath>
 
+#include "lanes.cuh"
+
 namespace mcrt {
 
 constexpr double kH = 6.62607015e-27;
@@ -120,19 +122,30 @@ __host__ __device__ inline void planck_bins(const double* lam_e, int nlam, doubl
   }
 }
 
-// Rosseland mean of chi' = kappa + (1-g) sigma at T (Eq. 3 with Eq. 16), exact bin integrals
-__host__ __device__ inline double rosseland(const double* lam_e, const double* chip, int nlam, double T) {
-  double g4p = 0.0, s1 = 0.0, s2 = 0.0;
-  for (int b = 0; b < nlam; ++b) {
-    double g3, g4;
-    if (b + 1 == nlam) tails(0.0, g3, g4);
-    else tails(kH * kC / (lam_e[b + 1] * 1e-4 * kKB * T), g3, g4);
-    const double db = g4 - g4p;
-    s1 += db;
-    s2 += db / chip[b];
-    g4p = g4;
+// Rosseland mean of chi' = kappa + (1-g) sigma at T (Eq. 3 with Eq. 16), exact bin integrals; the lanes of g take the bins
+// side by side (a bin's short edge is its neighbour lane's long one), the result is in all of them.
+template <class Group>
+__host__ __device__ inline double rosseland_group(const Group& g, const double* __restrict__ lam_e,
+                                                  const double* __restrict__ chip, int nlam, double T) {
+  const double hx = kH * kC / (1e-4 * kKB * T);
+  double s1 = 0.0, s2 = 0.0, g4p = 0.0;  // (the tail at the first bin's short edge, lambda -> 0, is 0)
+  for (int b0 = 0; b0 < nlam; b0 += g.size()) {
+    const int b = b0 + g.lane();
+    double g3, g4 = 0.0;
+    if (b < nlam) tails(b + 1 == nlam ? 0.0 : hx / lam_e[b + 1], g3, g4);
+    const double a4 = g.below(g4, g4p);
+    if (b < nlam) {
+      s1 += g4 - a4;
+      s2 += (g4 - a4) / chip[b];
+    }
+    g4p = g.last(g4);
   }
+  s1 = g.sum(s1);
+  s2 = g.sum(s2);
   return s1 / s2;
+}
+__host__ __device__ inline double rosseland(const double* lam_e, const double* chip, int nlam, double T) {
+  return rosseland_group(OneLane(), lam_e, chip, nlam, T);
 }
 
 }  // namespace mcrt

@@ -9,23 +9,32 @@
 
 namespace mcrt {
 
-// Q(T) and dQ/dT (erg s^-1 g^-1 and per K) from the bin integrals of Bbar and of T dBbar/dT
-__host__ __device__ inline void q_sum(const double* lam_e, const double* kabs, int nlam, double T, double& Q, double& dQ) {
-  const double k4 = kKB * kKB * kKB * kKB;
-  const double p3 = 2.0 * k4 * T * T * T * T / (kH * kH * kH * kC * kC);
-  const double p4 = 2.0 * k4 * T * T * T / (kH * kH * kH * kC * kC);
-  double g3p = 0.0, g4p = 0.0, s3 = 0.0, s4 = 0.0;
-  for (int b = 0; b < nlam; ++b) {
-    double g3, g4;
-    if (b + 1 == nlam) tails(0.0, g3, g4);
-    else tails(kH * kC / (lam_e[b + 1] * 1e-4 * kKB * T), g3, g4);
-    s3 += kabs[b] * (g3 - g3p);
-    s4 += kabs[b] * (g4 - g4p);
-    g3p = g3;
-    g4p = g4;
+// Q(T) and dQ/dT (erg s^-1 g^-1 and per K) from the bin integrals of Bbar and of T dBbar/dT; the lanes of g take the bins side
+// by side (a bin's short edge is its neighbour lane's long one), the result is in all of them.
+template <class Group>
+__host__ __device__ inline void q_sum_group(const Group& g, const double* __restrict__ lam_e, const double* __restrict__ kabs,
+                                            int nlam, double T, double& Q, double& dQ) {
+  const double pref = 8.0 * kPi * kKB * kKB * kKB * kKB / (kH * kH * kH * kC * kC);
+  const double hx = kH * kC / (1e-4 * kKB * T);
+  double s3 = 0.0, s4 = 0.0, g3p = 0.0, g4p = 0.0;  // sums over the bins of kappa dG3, kappa dG4
+  for (int b0 = 0; b0 < nlam; b0 += g.size()) {
+    const int b = b0 + g.lane();
+    double g3 = 0.0, g4 = 0.0;
+    if (b < nlam) tails(b + 1 == nlam ? 0.0 : hx / lam_e[b + 1], g3, g4);
+    const double a3 = g.below(g3, g3p), a4 = g.below(g4, g4p);
+    if (b < nlam) {
+      s3 += kabs[b] * (g3 - a3);
+      s4 += kabs[b] * (g4 - a4);
+    }
+    g3p = g.last(g3);
+    g4p = g.last(g4);
   }
-  Q = 4.0 * kPi * p3 * s3;
-  dQ = 4.0 * kPi * p4 * s4;
+  const double p3 = pref * T * T * T;
+  Q = p3 * T * g.sum(s3);
+  dQ = p3 * g.sum(s4);
+}
+__host__ __device__ inline void q_sum(const double* lam_e, const double* kabs, int nlam, double T, double& Q, double& dQ) {
+  q_sum_group(OneLane(), lam_e, kabs, nlam, T, Q, dQ);
 }
 
 // The T of the tabulated grid for Q(T) = q > 0 (lQk: log Q(T_k), slQ: d log Q / d log T at T_k, T_k = Tmin exp((k-1)
@@ -71,22 +80,27 @@ __host__ __device__ inline bool newton_step(double q, double Q, double dQ, doubl
   return fabs(xn - x) <= 1e-15 * x;
 }
 
-// T with Q(T) = q > 0: gray dust in closed form, otherwise bracketed Newton from the tabulated grid's T
-__host__ __device__ inline double cell_temperature(double q, int gray, double kabs0, int nlam, const double* lam_e,
-                                                   const double* kabs, const double* lQk, const double* slQ, int nT,
-                                                   double Tmin, double dlnT) {
-  if (gray) {
-    return pow(q / (4.0 * MCRT_SIGMA * kabs0), 0.25);
-  }
-  double lo = 0.0, hi = INFINITY, x = temperature_guess(q, lQk, slQ, nT, Tmin, dlnT);
+// T with Q(T) = q > 0 by bracketed Newton from x (the tabulated grid's T)
+template <class Group>
+__host__ __device__ inline double temperature_root(const Group& g, double q, double x, int nlam, const double* __restrict__ lam_e,
+                                                   const double* __restrict__ kabs) {
+  double lo = 0.0, hi = INFINITY;
   for (int it = 0; it < 100; ++it) {
     double Q, dQ, xn;
-    q_sum(lam_e, kabs, nlam, x, Q, dQ);
+    q_sum_group(g, lam_e, kabs, nlam, x, Q, dQ);
     const bool done = newton_step(q, Q, dQ, x, lo, hi, xn);
     x = xn;
     if (done) break;
   }
   return x;
+}
+
+// T with Q(T) = q > 0: gray dust in closed form
+__host__ __device__ inline double cell_temperature(double q, int gray, double kabs0, int nlam, const double* lam_e,
+                                                   const double* kabs, const double* lQk, const double* slQ, int nT,
+                                                   double Tmin, double dlnT) {
+  if (gray) return pow(q / (4.0 * MCRT_SIGMA * kabs0), 0.25);
+  return temperature_root(OneLane(), q, temperature_guess(q, lQk, slQ, nT, Tmin, dlnT), nlam, lam_e, kabs);
 }
 
 }  // namespace mcrt
