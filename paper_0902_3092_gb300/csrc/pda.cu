@@ -52,6 +52,7 @@ struct PdaState {
   DBuf sc;                            // FP64 CG scalars per iteration
   DBuf kctr;                          // int: index of the CG iteration, on the device (graph replay)
   DBuf red;                           // FP64 reduction slots
+  DBuf x0;                            // the box's cells before a cluster step
   DBuf w, gl, gk;                     // adjoint weights / gradient outputs (device staging)
   int n_pda = 0;
   int max_inner_alloc = 0;
@@ -536,6 +537,54 @@ __global__ void k_update(int n, const signed char* mask, const double* dis, cons
   if (c < n && mask[c] == 2) x[c] += scale * dis[c] * (double)y[c];
 }
 
+// k_update of a cluster solve; the cells' values before it are kept in x0 (box: rows from i0, w columns from j0)
+__global__ void k_update_keep(int n, int nt, const signed char* mask, const double* dis, const float* y, double scale, double* x,
+                              double* x0, int i0, int j0, int w) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n || mask[c] != 2) return;
+  const int i = c / nt, j = c - i * nt;
+  const double v = x[c];
+  x0[(size_t)(i - i0) * w + (j - j0)] = v;
+  x[c] = v + scale * dis[c] * (double)y[c];
+}
+
+// ... and back
+__global__ void k_take_back(int n, int nt, const signed char* mask, double* x, const double* x0, int i0, int j0, int w) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n || mask[c] != 2) return;
+  const int i = c / nt, j = c - i * nt;
+  x[c] = x0[(size_t)(i - i0) * w + (j - j0)];
+}
+
+// Where a refinement stands between its steps. The cluster solves (cgcluster.cuh) keep their scalars in floats and pairs of floats:
+// with neighbouring conductances that differ by 1e8 and more they may not reduce the residual, or end in no number (the
+// tile kernels' FP64 sums do better there). A step of theirs that does not halve it is the last one, and is taken back if it
+// made it worse; the tile kernels then refine what there is, with all of the caller's steps. The result is then
+// no further off than theirs from the start, and what they solve stays solved.
+struct Refinement {
+  bool cluster;
+  int steps = 0;         // made by the present kernels
+  double prev = INFINITY;  // residual before the last step
+  double best = INFINITY;
+  int stall = 0;
+  explicit Refinement(bool c) : cluster(c) {}
+  // the cluster's last step is not kept going on: the residual is rn now
+  bool cluster_ends(double rn, int max_steps) const {
+    return cluster && steps > 0 && (!(rn < 0.5 * prev) || steps == max_steps);
+  }
+  void to_tiles() { *this = Refinement(false); }
+  // FP64 rounding floor of the residual: no halving for three refinement steps below 1e-8
+  bool at_floor(double rn, double norm_b) {
+    if (rn < 0.5 * best) {
+      best = rn;
+      stall = 0;
+    } else if (++stall >= 3 && best <= 1e-8 * norm_b) {
+      return true;
+    }
+    return false;
+  }
+};
+
 __global__ void k_tpda(int n, const signed char* mask, const double* u, const double* Tmc, double* Tp) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
@@ -666,6 +715,7 @@ static mcrt_status pda_alloc(mcrt_disk* d, int max_inner) {
     for (DBuf* b : d4)
       if (e == cudaSuccess) e = b->alloc((size_t)n * 4);
     if (e == cudaSuccess) e = P->mask.alloc(n);
+    if (e == cudaSuccess) e = P->x0.alloc((size_t)std::min<long long>(n, kCgMaxCells) * 8);
     if (e == cudaSuccess) e = P->tiles.alloc(((size_t)n + 31) / 32 * sizeof(int));
     if (e == cudaSuccess) e = P->red.alloc(16 * 8);
     if (e == cudaSuccess) e = P->kctr.alloc(16);
@@ -768,8 +818,8 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
   const int* tiles = P->tiles.as<int>();
   const int ga = P->vec4 ? tgrid(k_cg_a4, P->ntiles) : tgrid(k_cg_a<kUA>, P->ntiles);
   const int gb = P->vec4 ? tgrid(k_cg_b4, P->ntiles) : tgrid(k_cg_b<kUB>, P->ntiles);
-  double norm_b = -1.0, best = INFINITY;
-  int total_iters = 0, stall = 0;
+  double norm_b = -1.0;
+  int total_iters = 0;
   constexpr int chunk = 32;
   // a region whose box fits one cluster is solved by one launch per refinement step (cgcluster.cuh)
   const CgBox box{nt, P->box[0], P->box[2], P->box[1] - P->box[0], P->box[3] - P->box[2], P->ar.as<float>(),
@@ -779,44 +829,56 @@ static mcrt_status refine_solve(mcrt_disk* d, const mcrt_pda_opts* o, double* x,
   // without a graph (capture refused, e.g. on the legacy default stream) the kernels launch one by one
   int* kdev = P->kctr.as<int>();
   ChunkGraph cg;
-  cudaGraphExec_t chunk_exec = plan.nc ? nullptr : cg.build(st, chunk, [&](int j) {
-    launch_cg_iteration(P, n, nt, tiles, r, pb[(j + 1) & 1], pb[j & 1], Ap, y, sc, kdev, 0, o->max_inner, tol2_in, ga,
-                        gb, st);
-    k_iter_next<<<1, 1, 0, st>>>(kdev);
-  });
-  for (int outer = 0; outer <= o->max_outer; ++outer) {
+  auto build_chunk = [&] {
+    return cg.build(st, chunk, [&](int j) {
+      launch_cg_iteration(P, n, nt, tiles, r, pb[(j + 1) & 1], pb[j & 1], Ap, y, sc, kdev, 0, o->max_inner, tol2_in, ga,
+                          gb, st);
+      k_iter_next<<<1, 1, 0, st>>>(kdev);
+    });
+  };
+  cudaGraphExec_t chunk_exec = plan.nc ? nullptr : build_chunk();
+  double* x0 = P->x0.as<double>();
+  for (Refinement ref(plan.nc > 0);; ++ref.steps) {
     CK(cudaMemsetAsync(red + 4, 0, 8, st), "memset");
     k_resid64<<<sgrid(n), 256, 0, st>>>(nr, nt, mask, Cr, Ct, dis, x, b, P->rs.as<double>(), red, 4);
     d->launches++;
     double rn2 = 0.0;
     int made = 0;  // iterations of the last cluster solve
     CK(cudaMemcpyAsync(&rn2, red + 4, 8, cudaMemcpyDeviceToHost, st), "copy");
-    if (plan.nc && outer > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
+    if (ref.cluster && ref.steps > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
     CK(cudaStreamSynchronize(st), "synchronize");
     total_iters += made;
     const double rn = std::sqrt(rn2);
     if (norm_b < 0) norm_b = rn;  // first residual: x = 0 on the PDA cells, so this is |S b_total|
-    if (!(rn == rn)) return set_error(d, MCRT_ENOTCONV, "PDA residual is not finite");
     if (rn <= o->tol * norm_b || rn == 0.0) {
       if (iters_out) *iters_out = total_iters;
       return MCRT_OK;
     }
-    // FP64 rounding floor of the residual: no halving for three refinement steps below 1e-8
-    if (rn < 0.5 * best) {
-      best = rn;
-      stall = 0;
-    } else if (++stall >= 3 && best <= 1e-8 * norm_b) {
+    if (ref.cluster_ends(rn, o->max_outer)) {
+      const bool worse = !(rn < ref.prev);
+      ref.to_tiles();
+      chunk_exec = build_chunk();
+      if (worse) {
+        k_take_back<<<nblk(n), 256, 0, st>>>(n, nt, mask, x, x0, box.i0, box.j0, box.w);
+        d->launches++;
+        ref.steps = -1;  // (the residual of x again)
+        continue;
+      }
+    }
+    if (!(rn == rn)) return set_error(d, MCRT_ENOTCONV, "PDA residual is not finite");
+    if (!ref.cluster && ref.at_floor(rn, norm_b)) {
       if (iters_out) *iters_out = total_iters;
       return MCRT_OK;
     }
-    if (outer == o->max_outer) break;
+    if (ref.steps == o->max_outer) break;
+    ref.prev = rn;
     const double scale = residual_scale(rn);
     // inner FP32 CG on the unit-diagonal system
-    if (plan.nc) {
+    if (ref.cluster) {
       CgBox b1 = box;
       b1.inv_scale = 1.0 / scale;
       CK(cg_solve(b1, plan, st), "PDA cluster kernel");
-      k_update<<<nblk(n), 256, 0, st>>>(n, mask, dis, y, scale, x);
+      k_update_keep<<<nblk(n), 256, 0, st>>>(n, nt, mask, dis, y, scale, x, x0, box.i0, box.j0, box.w);
       d->launches += 2;
       CK(cudaGetLastError(), "PDA kernels");
       continue;
@@ -1185,39 +1247,46 @@ extern "C" mcrt_status mcrt_pda_solve_static(int device, int nr, int ntheta, con
   const CgPlan plan = bx[1] ? cg_plan(box.rows, box.w, o->max_inner) : CgPlan();
   const int ntiles = (n + 31) / 32;  // every tile of the grid
   const int ga = tgrid(k_cg_a<kUA>, ntiles), gb = tgrid(k_cg_b<kUB>, ntiles);
-  double best = INFINITY;
-  int total_iters = 0, stall = 0;
+  int total_iters = 0;
   const int chunk = 32;
   double h[2 * chunk + 2];
-  for (int outer = 0; outer <= o->max_outer; ++outer) {
+  double* const x0 = reinterpret_cast<double*>(r);  // the box before a cluster step (r and p0, which only the tile kernels use)
+  for (Refinement ref(plan.nc > 0);; ++ref.steps) {
     CK(cudaMemsetAsync(red + 4, 0, sizeof(double), st), "memset");
     k_resid64<<<sgrid(n), 256, 0, st>>>(nr, nt, mask_dev, Cr_dev, Ct_dev, dis, u_dev, nullptr, rs, red, 4);
     double rn2 = 0.0;
     int made = 0;  // iterations of the last cluster solve
     CK(cudaMemcpyAsync(&rn2, red + 4, sizeof(double), cudaMemcpyDeviceToHost, st), "copy");
-    if (plan.nc && outer > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
+    if (ref.cluster && ref.steps > 0) CK(cudaMemcpyAsync(&made, kdev, sizeof(int), cudaMemcpyDeviceToHost, st), "copy");
     CK(cudaStreamSynchronize(st), "synchronize");
     total_iters += made;
     const double rn = std::sqrt(rn2);
-    if (!(rn == rn)) return set_error(nullptr, MCRT_ENOTCONV, "PDA residual is not finite");
     if (rn <= o->tol * norm_b || rn == 0.0) {
       if (out_iters) *out_iters = total_iters;
       return MCRT_OK;
     }
-    if (rn < 0.5 * best) {
-      best = rn;
-      stall = 0;
-    } else if (++stall >= 3 && best <= 1e-8 * norm_b) {
+    if (ref.cluster_ends(rn, o->max_outer)) {
+      const bool worse = !(rn < ref.prev);
+      ref.to_tiles();
+      if (worse) {
+        k_take_back<<<nblk(n), 256, 0, st>>>(n, nt, mask_dev, u_dev, x0, box.i0, box.j0, box.w);
+        ref.steps = -1;  // (the residual of u again)
+        continue;
+      }
+    }
+    if (!(rn == rn)) return set_error(nullptr, MCRT_ENOTCONV, "PDA residual is not finite");
+    if (!ref.cluster && ref.at_floor(rn, norm_b)) {
       if (out_iters) *out_iters = total_iters;
       return MCRT_OK;
     }
-    if (outer == o->max_outer) break;
+    if (ref.steps == o->max_outer) break;
+    ref.prev = rn;
     const double scale = residual_scale(rn);
-    if (plan.nc) {
+    if (ref.cluster) {
       CgBox b1 = box;
       b1.inv_scale = 1.0 / scale;
       CK(cg_solve(b1, plan, st), "PDA cluster kernel");
-      k_update<<<nblk(n), 256, 0, st>>>(n, mask_dev, dis, y, scale, u_dev);
+      k_update_keep<<<nblk(n), 256, 0, st>>>(n, nt, mask_dev, dis, y, scale, u_dev, x0, box.i0, box.j0, box.w);
       CK(cudaGetLastError(), "PDA kernels");
       continue;
     }
