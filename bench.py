@@ -43,14 +43,16 @@ WORKLOAD = "thick gray disk 200x120 rim-refined, tau_mid=1e6, albedo 0.5 isotrop
 # counts live in the profile summary written from that capture, so a kernel change without a new capture
 # leaves the roofline figures null.
 COUNTS_FILE = os.path.join(ROOT, "profiles", "transport_counts_thickgray_200x120.md")
+# The same for the ray-tracing kernel: counts per ray segment through dust of the 200x120 disk at 45 degrees, 100 bins.
+RAY_COUNTS_FILE = os.path.join(ROOT, "profiles", "raytrace_thickgray_200x120_ncu.md")
 N_SMS, SCHEDULERS = 152, 4
 
 
-def transport_counts():
-    """Per-step counts of the profile summary: the indented `key: value` lines."""
+def transport_counts(path=None):
+    """Counts of a profile summary (the transport's): the indented `key: value` lines."""
     out = {}
     try:
-        with open(COUNTS_FILE) as f:
+        with open(path or COUNTS_FILE) as f:
             for ln in f:
                 m = re.match(r"^    ([a-z0-9_]+): (\S+)\s*$", ln)
                 if m:
@@ -86,15 +88,41 @@ def code_only(src):
     return " ".join("".join(out).split())
 
 
-def transport_source_hash(root=None):
+def transport_source_hash(root=None, files=("common.cuh", "transport.cuh", "transport_f32.cu")):
     """Hash of the transport kernels' code (comments and layout left out): counts taken from another
     version of the code are not used."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("common.cuh", "transport.cuh", "transport_f32.cu"):
+    for f in files:
         with open(os.path.join(root or ROOT, "paper_0902_3092_gb300", "csrc", f), encoding="utf-8") as fh:
             h.update(code_only(fh.read()).encode())
     return h.hexdigest()[:16]
+
+
+def ray_source_hash(root=None):
+    """The same of the ray-tracing kernel's code."""
+    return transport_source_hash(root, ("common.cuh", "raymarch.cuh", "raytrace.cu"))
+
+
+def ray_roofline(segments, t_call, sm_mhz):
+    """Issue-slot roofline of one mcrt_raytrace call: the ray-tracing kernel's warp instructions per segment (ncu) x the
+    call's segments / its CUDA-event time, against 152 SMs x 4 schedulers x the SM clock."""
+    c = transport_counts(RAY_COUNTS_FILE)
+    peak = N_SMS * SCHEDULERS * sm_mhz * 1e6
+    roof = {"bound": "alu", "unit": "warp-inst/s", "peak": peak, "achieved": None, "frac": None, "traffic": None,
+            "thread_inst_frac": None, "kernel": "k_raytrace<float, 4> (time: with k_sed_part and k_sed_final)",
+            "counts_file": os.path.relpath(RAY_COUNTS_FILE, ROOT)}
+    if c.get("source_sha16") != ray_source_hash():
+        roof["note"] = "no ncu counts for the current ray-tracing kernel (its sources changed since the capture)"
+        return roof
+    wps, tps = c["warp_inst_per_segment"], c["thread_inst_per_segment"]
+    ach = wps * segments / t_call
+    roof.update({"achieved": ach, "frac": ach / peak, "traffic": c["dram_bytes_per_launch"],
+                 "thread_inst_frac": tps * segments / t_call / (32 * peak),
+                 "note": f"issue slots: {wps:.1f} warp instructions per segment through dust (ncu) x {segments} segments / "
+                         f"CUDA-event call time; peak = 152 SMs x 4 schedulers x {sm_mhz:g} MHz; thread_inst_frac counts "
+                         "active lanes"})
+    return roof
 
 
 def transport_roofline(steps_per_launch, t_launch, clocks, peaks):
@@ -574,15 +602,6 @@ def pda_adjoint_timing(args):
     print(json.dumps(line), flush=True)
 
 
-# issue-slot work of the ray-tracing kernel: warp instructions per ray segment through dust (ncu
-# smsp__inst_executed of k_raytrace<float, 25> on the 200x120 disk at 45 degrees, 2.765e9, over its
-# 17,980,808 segments; the count includes the crossings of dust-free cells, 40 % of all crossings, and
-# the four marches of each ray, one per chunk of 25 wavelength bins)
-RAY_WARP_INST_PER_SEG = 153.8
-RAY_THREAD_INST_PER_SEG = 2835.5  # smsp__thread_inst_executed (5.098e10) over the same segments
-RAY_DRAM_BYTES = 14522624 + 6551040  # dram__bytes_read.sum + dram__bytes_write.sum of the same launch
-
-
 def raytrace_timing(args):
     """Ray-traced SED and image (Sect. 2.3, 4.1) of the 200 x 120 rim-refined tau_mid = 1e6 gray disk at 45
     degrees and 140 pc, after a 1e7-packet MRW run (Monte Carlo temperatures): 104,448 rays (16 rings
@@ -633,18 +652,7 @@ def raytrace_timing(args):
     t_e2e = float(np.median(e2e))
     peaks = measured_peaks()
     clocks = clk.summary()
-    mhz = clocks["sm_mhz"] or 2070.0
-    issue_peak = 152 * 4 * mhz * 1e6
-    roof = {"bound": "alu", "unit": "warp-inst/s", "kernel": "k_raytrace<float, 25> (+ k_star, k_sed_part, k_sed_final)"}
-    if RAY_WARP_INST_PER_SEG:
-        ach = RAY_WARP_INST_PER_SEG * seg / t
-        roof.update({"achieved": ach, "peak": issue_peak, "frac": ach / issue_peak, "traffic": RAY_DRAM_BYTES,
-                     "thread_inst_frac": RAY_THREAD_INST_PER_SEG * seg / t / (32 * issue_peak),
-                     "note": f"issue-slot roofline: {RAY_WARP_INST_PER_SEG} warp instructions per segment (ncu) x "
-                             f"{seg} segments / CUDA-event call time; peak = 152 SMs x 4 schedulers x SM clock; "
-                             "thread_inst_frac counts active lanes"})
-    else:
-        roof.update({"achieved": None, "peak": issue_peak, "frac": None, "traffic": None})
+    roof = ray_roofline(seg, t, clocks["sm_mhz"] or 2070.0)
     # the oracle on the host cores: rays one by one for about ten seconds
     cpu = None
     if not args.no_cpu:
@@ -669,7 +677,7 @@ def raytrace_timing(args):
                        "rays": rays.n, "wavelength_bins": n_bins, "segments": seg, "l2": "flushed (256 MB write)"},
             "e2e": {"value": rays.n / t_e2e, "unit": "rays/s", "h2d_bytes_per_step": 3 * 8 * rays.n,
                     "d2h_bytes_per_step": 16 * n_bins},
-            "roofline": roof, "cpu_baseline": cpu, "clocks": clocks, "gpu_launches": 4,
+            "roofline": roof, "cpu_baseline": cpu, "clocks": clocks, "gpu_launches": 3 * args.steps,
             "flux_total_erg_s_cm2": float(out["F"].sum())}
     if scat:
         line["config"]["scattering"] = "mean-intensity tally, sigma J / chi in the source function"
