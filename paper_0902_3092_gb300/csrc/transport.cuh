@@ -1345,6 +1345,12 @@ __device__ __forceinline__ void flush(const DevModel<R>& M, Acc& acc, bool warp_
   acc = Acc{};
 }
 
+// ... before a counter of one that carries packet after packet (a warp of few in flight may make a whole run) gets near 2^32
+template <class R>
+__device__ __forceinline__ void flush_if_full(const DevModel<R>& M, Acc& acc) {
+  if ((acc.cross | acc.sca | acc.abs | acc.mrw) >> 30) flush(M, acc, false);
+}
+
 // model of queue position q (batch launches): largest m with q_begin <= q
 template <class R>
 __device__ __forceinline__ int find_model(const KParams<R>& P, unsigned long long q) {
@@ -1978,6 +1984,7 @@ __global__ void __launch_bounds__(32, kWarpBlocksPerSm) transport_warp_kernel(co
     if (lane == 0) {
       note_end(s, acc);
       if (BATCH) flush(M, acc, false);
+      else flush_if_full(M, acc);
     }
     if (BATCH) acc = Acc{};
   }

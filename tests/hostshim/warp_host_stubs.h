@@ -28,6 +28,12 @@
 #undef __reduce_or_sync
 #undef __syncwarp
 
+inline unsigned long long atomicOr(unsigned long long* p, unsigned long long v) {
+  const unsigned long long o = *p;
+  *p |= v;
+  return o;
+}
+
 class HostWarp {
  public:
   // body(lane) in 32 lanes; false: the lanes parted

@@ -157,3 +157,25 @@ extern "C" int host_warp_transport(int nr, int nt, const double* rf_cm, const do
   for (int i = 0; i < 8; ++i) counters[i] = c[i];
   return ok ? 0 : 1;
 }
+
+// The run counters (C_NCNT values) after `times` packets of the given counts, kept as the kernel keeps them (and flushed at its end).
+extern "C" void host_counters(int times, unsigned cross, unsigned sca, unsigned abs, unsigned mrw, uint64_t* cnt) {
+  DevModel<float> M;
+  std::memset(&M, 0, sizeof(M));
+  M.cnt = (unsigned long long*)cnt;
+  Acc acc;
+  std::memset(&acc, 0, sizeof(acc));
+  for (int k = 0; k < times; ++k) {
+    acc.cross += cross;
+    acc.sca += sca;
+    acc.abs += abs;
+    acc.mrw += mrw;
+    acc.packets++;
+    flush_if_full(M, acc);
+  }
+  flush(M, acc, false);
+}
+extern "C" void host_counter_places(int* at) {
+  const int p[5] = {C_PACKETS, C_CROSS, C_SCA, C_ABS, C_MRW};
+  for (int i = 0; i < 5; ++i) at[i] = p[i];
+}

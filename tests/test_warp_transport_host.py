@@ -60,3 +60,12 @@ def test_lanes_agree_on_a_tally_that_other_packets_change(lib, form):
         assert np.array_equal(a[k], b[k]), k
     if a["j"] is not None:
         assert np.array_equal(a["j"], b["j"])
+
+
+def test_counters_of_a_long_run_do_not_wrap(lib):
+    """A warp that makes a run's packets one after another passes 2^32 crossings."""
+    each, times = (700_000_000, 90_000_000, 80_000_000, 3), 60
+    cnt, at = np.zeros(64, np.uint64), np.zeros(5, np.int32)
+    lib.host_counter_places(at.ctypes.data_as(C.c_void_p))
+    lib.host_counters(C.c_int(times), *(C.c_uint(x) for x in each), cnt.ctypes.data_as(C.c_void_p))
+    assert [int(cnt[i]) for i in at] == [times] + [times * x for x in each]
