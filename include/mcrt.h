@@ -154,7 +154,7 @@ typedef struct {
   uint64_t guarded;           /* packets dropped by a step guard */
   uint64_t guard_packet;      /* full id of the first of them */
   int32_t guard_kind;         /* 0 none, 1 step limit, 2 face crossings without an interaction */
-  int32_t guard_in_tail;      /* 1 if the tail kernel carried it */
+  int32_t guard_in_tail;      /* 1 if a warp carried it alone (the tail kernel, or a run of such packets) */
   int32_t guard_cell[2];      /* its cell (ir, itheta) when the guard fired; ir = -1: inner cavity */
   uint64_t guard_events, guard_steps;  /* its interactions + jumps and its steps then */
   double guard_pos_cm[3];     /* its position (cm) and direction then */

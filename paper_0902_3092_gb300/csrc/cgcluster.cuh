@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(cg_threads(K), 1) k_cg_cluster(const CgBox B) 
 // lanes' affine maps by shuffle (their multipliers are constants, kept in shared memory), E more to add the carry;
 // no barrier. The two neighbour rows are solved here too. Odd E keeps the lanes' shared-memory accesses free of bank
 // conflicts (E = 2: two-way). An iteration costs 2.9 us against 2.1; whole solves, diagonal -> line: PDA of the 400x200
-// disk 5.25 -> 3.97 ms (at the full residual, kCgStop = 1, as the others), of a 200x120 disk 1.19 -> 0.75, equal couplings 98x58 0.89 -> 0.85, 198x118 2.06 -> 1.83,
+// disk 5.25 -> 3.97 ms (at the full residual, kCgStop = 1, as the others), of a 200x120 disk 1.19 -> 0.75, equal
+// couplings 98x58 0.89 -> 0.85, 198x118 2.06 -> 1.83,
 // 98x278 3.12 -> 2.44, 22x18 0.31 -> 0.33, 298x10 0.47 -> 0.53 (iterations of the diagonal one on strong couplings pay
 // for those two many times over).
 constexpr int kScan = 10;  // scan multipliers per row and lane: five steps forward, five backward

@@ -224,11 +224,11 @@ __global__ void k_scaled(int nr, int nt, const signed char* mask, const double* 
 }
 
 // --------------------------------------------------------------------------------------------- FP64
-// rs = S (b + sum_f C_f (x_nb - x_c)) on PDA cells; red[slot] += |rs|^2
 // The factor that takes an inner right-hand side to FP32: a power of two, so that the last bits of rn (its blocks' sums are
 // added in any order) do not reach the FP32 solve: the same system gives the same solution.
 static double residual_scale(double rn) { return std::ldexp(1.0, std::ilogb(rn)); }
 
+// rs = S (b + sum_f C_f (x_nb - x_c)) on PDA cells; red[slot] += |rs|^2
 __global__ void k_resid64(int nr, int nt, const signed char* __restrict__ mask, const double* __restrict__ Cr,
                           const double* __restrict__ Ct, const double* __restrict__ dis, const double* __restrict__ x,
                           const double* __restrict__ b, double* __restrict__ rs, double* red, int slot) {

@@ -2,8 +2,9 @@
 //
 // int_bin B_nu(T) dnu = (2 k^4 T^4 / (h^3 c^2)) [F3(x_hi) - F3(x_lo)],  F3(x) = int_0^x t^3/(e^t-1) dt,
 // int_bin dB_nu/dT dnu = (2 k^4 T^3 / (h^3 c^2)) [F4(x_hi) - F4(x_lo)], F4(x) = int_0^x t^4 e^t/(e^t-1)^2 dt,
-// with x = h nu / (k T). For x <= 2, F3 is the power series of the Bernoulli numbers (Abramowitz & Stegun 27.1.1 for n = 3;
-// convergent for x < 2 pi, 17 terms leave 1e-17 at x = 2), and so is F4 = 4 F3 - x^4/(e^x - 1) (by parts); above, the complement int_x^inf t^3/(e^t - 1) dt is summed over int t^3 e^{-nt} dt (27.1.2).
+// with x = h nu / (k T). For x <= 2, F3 is the power series of the Bernoulli numbers (Abramowitz & Stegun 27.1.1 for
+// n = 3; convergent for x < 2 pi, 17 terms leave 1e-17 at x = 2), and so is F4 = 4 F3 - x^4/(e^x - 1) (by parts); above,
+// the complement int_x^inf t^3/(e^t - 1) dt is summed over int t^3 e^{-nt} dt (27.1.2).
 // The first bin extends to lambda -> 0 and the last to infinity.
 //
 // FP64 arithmetic bounds the kernels that use them (1.25 TFLOP/s on this GPU): about 25 operations per edge against
