@@ -11,7 +11,8 @@
 // recurrence s = A r + beta s. The barrier that brings the sums also brings A r of the neighbour CTAs' rows beside this CTA's,
 // whose r it updates itself. (With a barrier each for p.Ap and r.r a whole solve of the 400x200 disk's PDA took 6.4 ms
 // against 5.2.) The sums are FP32 in a CTA, the CTAs' sums pairs of floats (FP64 adds and divides have several times
-// the latency here), in a fixed order: the same system gives the same bits. Cells of the box that are no unknowns have zero
+// the latency here), in a fixed order: the same system gives the same bits. (Systems of very high contrast that this does
+// not carry are left to the tile kernels: Refinement in pda.cu.) Cells of the box that are no unknowns have zero
 // couplings and a zero right-hand side, and stay zero.
 //
 // Limit: about 100 rows of 32 columns to 14 of 288 per CTA with the line preconditioner, else 8192 cells per CTA; beyond it

@@ -1951,8 +1951,8 @@ constexpr int kWarpBlocksPerSm = 16;
 // waited for its 31 divergent neighbours (2.3 us a step); alone in a warp it waits for nobody, its flights
 // cross up to 31 cells in about the latency of two crossings, and its table searches take two dependent
 // loads. Measured (reset, run, temperatures, spectrum): 100x60 non-gray disk, tau_mid 1e5, MRW, 1e6 packets
-// 894 -> 222 ms (of which ~150 ms are its longest packets, ~7e4 steps of 2 us); 40x30, tau_mid 1e3, 1e6 packets
-// 160 -> 14.4 ms; a batch of six disks, 1.2e6 packets, 265 -> 19.8 ms. Runs that may have many more
+// 894 -> 301 ms (a third as many packets in flight as in lanes, see warp_grid; 222 with as many, of which ~150 ms are
+// its longest packets, ~7e4 steps of 2 us); 40x30, tau_mid 1e3, 1e6 packets 160 -> 16 ms; a batch of six disks, 1.2e6 packets, 265 -> 19.8 ms. Runs that may have many more
 // packets in flight than the device holds warps keep a packet per lane (see one_packet_per_warp).
 template <bool BATCH, bool JT>
 __global__ void __launch_bounds__(32, kWarpBlocksPerSm) transport_warp_kernel(const KParams<float> P) {
